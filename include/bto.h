@@ -372,10 +372,11 @@ BTO_API bto_status bto_stitch_pathlines_ex(const int32_t lattice[3], const float
  * The basis flow of a particle is a function of its start position and of
  * every cycle's node velocities (Sec. 3.1 advection, Eq. 1 sampling). A tape
  * runs one interval of one block from caller-given start positions, keeps
- * positions every checkpoint_every cycles, and then returns vector-Jacobian
- * products of the end positions: with respect to the start positions (the
- * flow-map Jacobian, from which FTLE) and to the node velocities. Segments
- * between checkpoints are recomputed during the backward sweep.
+ * positions at the start of segments of 1.2 sqrt(cycles) cycles (at least 4),
+ * and then returns vector-Jacobian products of the end positions: with
+ * respect to the start positions (the flow-map Jacobian, from which FTLE) and
+ * to the node velocities. The segments are recomputed, all at once, by a
+ * backward call.
  * A terminated particle's end is its last in-block position; its gradient
  * flows back through the cycles before its exit cycle only (termination
  * itself is a discrete decision with no gradient). Particles occupy fixed
@@ -384,8 +385,10 @@ BTO_API bto_status bto_stitch_pathlines_ex(const int32_t lattice[3], const float
 typedef struct bto_tape bto_tape;
 
 /* extent_cells, origin, spacing as in bto_create; num_particles >= 1;
- * cycles >= 1; checkpoint_every >= 1 (clamped to cycles). Allocates
- * (cycles/checkpoint_every + 2 + checkpoint_every) * num_particles * 16 B. */
+ * cycles >= 1; checkpoint_every >= 1 (checked, and otherwise without effect:
+ * the segments follow from the cycles alone, so results do not depend on it).
+ * Allocates (52 * segments + 8) * num_particles + 131,072 bytes, about
+ * 43 sqrt(cycles) bytes a particle. */
 BTO_API bto_status bto_tape_create(const int32_t extent_cells[3], const float origin[3],
                                    const float spacing[3], int64_t num_particles,
                                    int32_t cycles, int32_t checkpoint_every, bto_tape **out);
@@ -403,7 +406,7 @@ BTO_API bto_status bto_tape_forward(bto_tape *tape, const float *d_seeds,
                                     const void *const *d_field_table, float dt, float *d_ends,
                                     uint8_t *d_valid, int32_t *d_exit_cycle, bto_stream stream);
 
-/* Reverse sweep of the last forward.
+/* Gradients of the last forward.
  *   d_grad_ends          P*3 floats: dL/d(end position)
  *   d_grad_seeds         P*3 floats written: dL/d(start position)
  *   d_grad_field_table   NULL, or DEVICE array of `cycles` device pointers to
@@ -415,7 +418,7 @@ BTO_API bto_status bto_tape_backward(bto_tape *tape, const float *d_grad_ends,
                                      bto_stream stream);
 
 /* Flow-map Jacobian of the last forward: d_jac (P*9 floats, row-major per
- * particle) receives J[a][b] = d end_a / d start_b (three reverse sweeps). */
+ * particle) receives J[a][b] = d end_a / d start_b. */
 BTO_API bto_status bto_tape_jacobian(bto_tape *tape, float *d_jac, bto_stream stream);
 
 /* FTLE from a Jacobian: d_ftle[p] = ln(sqrt(lambda_max(J^T J))) / |cycles*dt|
