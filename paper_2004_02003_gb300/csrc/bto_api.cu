@@ -563,6 +563,23 @@ bto_status advect_ingest(bto_ctx *c, const void *field, const void *const *field
     return BTO_OK;
 }
 
+bto::AdvectArgs advect_args(const bto_ctx *c, const void *field, const void *const *fields, float dt) {
+    bto::AdvectArgs a{};
+    a.blocks = c->blocks;
+    a.gblock = c->gblock;
+    a.nb = c->nb;
+    a.cycle = c->cycle;
+    a.field = field;
+    a.fields = fields;
+    a.p = part_list(c);
+    a.err = c->derr;
+    a.ngroups = c->slots / group_size(c);
+    a.term = c->term;
+    a.clip = c->clip;
+    a.dt = dt;
+    return a;
+}
+
 bto_status advect_impl(bto_ctx *c, const void *field, const void *const *fields, float dt,
                        cudaStream_t s) {
     if (!std::isfinite(dt)) return BTO_ERR_INVALID_ARG;
@@ -617,19 +634,7 @@ bto_status advect_impl(bto_ctx *c, const void *field, const void *const *fields,
         c->cycle = cyc + 1;
         return BTO_OK;
     }
-    bto::AdvectArgs a{};
-    a.blocks = c->blocks;
-    a.gblock = c->gblock;
-    a.nb = c->nb;
-    a.cycle = cyc;
-    a.field = field;
-    a.fields = fields;
-    a.p = part_list(c);
-    a.err = c->derr;
-    a.ngroups = c->slots / group_size(c);
-    a.term = c->term;
-    a.clip = c->clip;
-    a.dt = dt;
+    const bto::AdvectArgs a = advect_args(c, field, fields, dt);
     cudaError_t e = bto::launch_advect(a, c->layout, c->nt, c->ppt, c->cap, c->grid, c->dyn_smem, s);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
@@ -729,6 +734,17 @@ bto_status bto_launch_interval_graph(bto_ctx *ctx, const void *const *d_field_ta
     if (reinterpret_cast<uintptr_t>(d_field_table) % alignof(void *)) return BTO_ERR_INVALID_ARG;
     if (ctx->cycle != 0) return BTO_ERR_STATE;
     if (ctx->ingest) return BTO_ERR_UNSUPPORTED;
+    if (!ctx->tiled) {
+        const cudaError_t e = bto::launch_interval(advect_args(ctx, nullptr, d_field_table, dt), ctx->layout, ctx->L,
+                                                   ctx->slots, group_size(ctx), (cudaStream_t)stream);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            ctx->sticky = cuda_status(e);
+            return ctx->sticky;
+        }
+        ctx->cycle = ctx->L;
+        return BTO_OK;
+    }
     const bool same = ctx->gexec && ctx->gtable == d_field_table && ctx->gdt == dt &&
                       ctx->gshape[0] == ctx->layout && ctx->gshape[1] == ctx->nt &&
                       ctx->gshape[2] == ctx->ppt && ctx->gshape[3] == ctx->grid &&
