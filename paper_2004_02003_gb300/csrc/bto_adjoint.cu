@@ -23,7 +23,8 @@
 // on 2 x 4 x 200 dependent samples. Measured on 64^3 cells: the Jacobian of
 // 100,003 particles over 50 cycles 2.43 -> 0.20 ms (three serial sweeps
 // against tangents and product), the gradients of 32,768 over 200 cycles
-// 1.97 -> 1.65 ms (0.24 tangents, 0.06 chain, 1.35 scatter).
+// 1.97 -> 1.08 ms (0.24 tangents, 0.01 chain, 0.83 scatter). Tangents and
+// scatter are bound by the L1 load path (73-74% of its wavefront peak).
 // A terminated particle's end is its last in-block position, so its gradient
 // flows back only through the cycles before its exit cycle.
 //
@@ -167,22 +168,18 @@ __global__ void tape_bin_kernel(const BlockDev *__restrict__ blk, int64_t P, con
 }
 
 // Step 2, one CTA: exclusive sums of the counts; the counts are left zero
-// for the next call.
-__global__ void __launch_bounds__(1024) tape_scan_kernel(int32_t *__restrict__ count, int32_t *__restrict__ start,
-                                                         int nbins) {
+// for the next call. 16-byte accesses: a thread's 16 bins are consecutive.
+__global__ void __launch_bounds__(1024) tape_scan_kernel(int4 *__restrict__ count, int4 *__restrict__ start) {
     __shared__ int32_t part[32];
-    constexpr int kPer = kMaxBins / 1024;
+    constexpr int kPer = kMaxBins / 4096;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int32_t v[kPer], sum = 0;
+    int4 v[kPer];
+    int32_t sum = 0;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        const int b = threadIdx.x * kPer + k;
-        v[k] = 0;
-        if (b < nbins) {
-            v[k] = count[b];
-            count[b] = 0;
-        }
-        sum += v[k];
+        v[k] = count[threadIdx.x * kPer + k];
+        count[threadIdx.x * kPer + k] = make_int4(0, 0, 0, 0);
+        sum += v[k].x + v[k].y + v[k].z + v[k].w;
     }
     int32_t incl = sum;
 #pragma unroll
@@ -196,9 +193,9 @@ __global__ void __launch_bounds__(1024) tape_scan_kernel(int32_t *__restrict__ c
     for (int w = 0; w < warp; ++w) run += part[w];
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        const int b = threadIdx.x * kPer + k;
-        if (b < nbins) start[b] = run;
-        run += v[k];
+        const int4 c = v[k];
+        start[threadIdx.x * kPer + k] = make_int4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
+        run += c.x + c.y + c.z + c.w;
     }
 }
 
@@ -251,10 +248,7 @@ __global__ void __launch_bounds__(kThreads) tape_forward_kernel(
                     left = C;
                 }
                 --left;
-                if (c + 1 < L) {
-                    next = table[c + 1];
-                    prefetch_cell<bto::LAYOUT_F3>(next, g, x);
-                }
+                if (c + 1 < L) next = table[c + 1];
                 if (rk4_step<bto::LAYOUT_F3>(x, field, g, s, q) != 0) {
                     e = c;
                     break;
@@ -271,90 +265,117 @@ __global__ void __launch_bounds__(kThreads) tape_forward_kernel(
     }
 }
 
-// Node-velocity gradients of one reverse cycle: stage k adds w_k(corner) g_k
-// to the 8 corners of its cell. Stages whose points lie in the same cell are
-// summed per corner first, so that each distinct cell takes 24 atomic adds
-// (the stages of a step mostly share a cell).
-__device__ __forceinline__ float stage_w(const Stage &st, int a, int b, int c) {
-    return (a ? st.fx : 1.f - st.fx) * (b ? st.fy : 1.f - st.fy) * (c ? st.fz : 1.f - st.fz);
+// Adds the corner gradients v[a + 2b + 4c] of the cell at `node` to gF: each
+// x-row of two nodes is six consecutive floats, added as pairs where the
+// address allows it (4-byte aligned: three pairs, or two pairs between two
+// single words), 14 atomic operations a cell on average instead of 24.
+__device__ __forceinline__ void red2(float *p, float a, float b) {
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
 }
-
-__device__ __forceinline__ void scatter_step(float *__restrict__ gF, const Geo &g, const Stage (&st)[4],
-                                             const float3 (&gs)[4]) {
-    unsigned done = 0;
+__device__ __forceinline__ void add_cell(float *__restrict__ gF, const Geo &g, uint32_t node, const float (&v)[8][3]) {
 #pragma unroll
-    for (int k = 3; k >= 0; --k) {
-        if (done & (1u << k)) continue;
-        bool in[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            in[j] = j <= k && !(done & (1u << j)) && st[j].ix == st[k].ix && st[j].iy == st[k].iy &&
-                    st[j].iz == st[k].iz;
-            if (in[j]) done |= 1u << j;
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
+        float *p = gF + 3ull * nd;
+        const float *a = v[2 * q], *b = v[2 * q + 1];
+        const bool odd = (reinterpret_cast<uintptr_t>(p) & 4u) != 0;
+        red2(p + (odd ? 1 : 0), odd ? a[1] : a[0], odd ? a[2] : a[1]);
+        red2(p + (odd ? 3 : 2), odd ? b[0] : a[2], odd ? b[1] : b[0]);
+        if (odd) {
+            atomicAdd(p, a[0]);
+            atomicAdd(p + 5, b[2]);
+        } else {
+            red2(p + 4, b[1], b[2]);
         }
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    float vx = 0.f, vy = 0.f, vz = 0.f;
-#pragma unroll
-                    for (int j = 3; j >= 0; --j) {
-                        if (!in[j]) continue;
-                        const float w = stage_w(st[j], a, b, c);
-                        vx = fmaf(w, gs[j].x, vx);
-                        vy = fmaf(w, gs[j].y, vy);
-                        vz = fmaf(w, gs[j].z, vz);
-                    }
-                    const uint32_t node = (uint32_t)(st[k].ix + a) + g.nnx * (uint32_t)(st[k].iy + b) +
-                                          g.nnxy * (uint32_t)(st[k].iz + c);
-                    float *p = gF + 3ull * node;
-                    atomicAdd(p + 0, vx);
-                    atomicAdd(p + 1, vy);
-                    atomicAdd(p + 2, vz);
-                }
     }
 }
 
-// Reverse of one cycle for one particle at xc (cell units) with adjoint lm
+// The cell of x (a point of the closed box), its corners from the cache or
+// the field, and x's fractions in it.
+__device__ __forceinline__ void locate(JCell &C, const float *__restrict__ f, const Geo &g, const float3 x, float &fx,
+                                       float &fy, float &fz) {
+    int ix, iy, iz;
+    cell_coord(x.x, g.cmx, ix, fx);
+    cell_coord(x.y, g.cmy, iy, fy);
+    cell_coord(x.z, g.cmz, iz, fz);
+    const uint32_t node = (uint32_t)ix + g.nnx * (uint32_t)iy + g.nnxy * (uint32_t)iz;
+    if (node != C.node) {
+        load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, ix, iy, iz, C.v);
+        C.node = node;
+    }
+}
+
+// (p - q) . w
+__device__ __forceinline__ float diff_dot(const float (&p)[3], const float (&q)[3], const float3 w) {
+    return fmaf(p[2] - q[2], w.z, fmaf(p[1] - q[1], w.y, (p[0] - q[0]) * w.x));
+}
+
+// (dv/dxi)^T w in the cell C at fractions (fx, fy, fz): the differences of
+// the corners along each axis, dotted with w and blended along the other two.
+__device__ __forceinline__ float3 grad_dot(const JCell &C, float fx, float fy, float fz, const float3 w) {
+    const float (&c)[8][3] = C.v;
+    return make_float3(
+        lerp1(lerp1(diff_dot(c[1], c[0], w), diff_dot(c[3], c[2], w), fy),
+              lerp1(diff_dot(c[5], c[4], w), diff_dot(c[7], c[6], w), fy), fz),
+        lerp1(lerp1(diff_dot(c[2], c[0], w), diff_dot(c[3], c[1], w), fx),
+              lerp1(diff_dot(c[6], c[4], w), diff_dot(c[7], c[5], w), fx), fz),
+        lerp1(lerp1(diff_dot(c[4], c[0], w), diff_dot(c[5], c[1], w), fx),
+              lerp1(diff_dot(c[6], c[2], w), diff_dot(c[7], c[3], w), fx), fy));
+}
+
+// Reverse of one cycle for one particle at x (cell units) with adjoint lm
 // (see the header of this file); adds the node-velocity gradients to gF.
-// Returns the adjoint before the cycle.
+// Returns the adjoint before the cycle. The stage points are found first;
+// then the stages are taken in reverse, their corners mostly still cached,
+// and the corner gradients of stages in one cell are summed before they are
+// added. No stage's Jacobian is formed: four of them held 36 registers and
+// left 12 warps per SM (32,768 particles over 200 cycles of 64^3 cells, with
+// scalar atomics: 1353 us; so, with paired ones: 831 us).
 __device__ __forceinline__ float3 adj_step(const float *__restrict__ f, float *__restrict__ gF, const Geo &g,
-                                           const float3 s, const float3 r, const float3 Lm) {
-    float3 k1, k2, k3, k4;
-    float J1[3][3], J2[3][3], J3[3][3], J4[3][3];
-    Stage st[4];
+                                           const float3 s, const float3 x, const float3 lm) {
     JCell C;
     C.node = ~0u;
-    sample_jac(C, f, g, r.x, r.y, r.z, k1, J1, st[0]);
-    sample_jac(C, f, g, fmaf(0.5f * s.x, k1.x, r.x), fmaf(0.5f * s.y, k1.y, r.y), fmaf(0.5f * s.z, k1.z, r.z),
-               k2, J2, st[1]);
-    sample_jac(C, f, g, fmaf(0.5f * s.x, k2.x, r.x), fmaf(0.5f * s.y, k2.y, r.y), fmaf(0.5f * s.z, k2.z, r.z),
-               k3, J3, st[2]);
-    sample_jac(C, f, g, fmaf(s.x, k3.x, r.x), fmaf(s.y, k3.y, r.y), fmaf(s.z, k3.z, r.z), k4, J4, st[3]);
-    const float3 s6 = make_float3(s.x / 6.f, s.y / 6.f, s.z / 6.f);
-    const float3 s3v = make_float3(s.x / 3.f, s.y / 3.f, s.z / 3.f);
-    float3 gs[4];
-    gs[0] = make_float3(s6.x * Lm.x, s6.y * Lm.y, s6.z * Lm.z);
-    gs[1] = make_float3(s3v.x * Lm.x, s3v.y * Lm.y, s3v.z * Lm.z);
-    gs[2] = gs[1];
-    gs[3] = gs[0];
-    float3 lx = Lm;
-    float3 q = jt_times(J4, gs[3]);
-    lx.x += q.x; lx.y += q.y; lx.z += q.z;
-    gs[2].x = fmaf(s.x, q.x, gs[2].x); gs[2].y = fmaf(s.y, q.y, gs[2].y); gs[2].z = fmaf(s.z, q.z, gs[2].z);
-    q = jt_times(J3, gs[2]);
-    lx.x += q.x; lx.y += q.y; lx.z += q.z;
-    gs[1].x = fmaf(0.5f * s.x, q.x, gs[1].x); gs[1].y = fmaf(0.5f * s.y, q.y, gs[1].y);
-    gs[1].z = fmaf(0.5f * s.z, q.z, gs[1].z);
-    q = jt_times(J2, gs[1]);
-    lx.x += q.x; lx.y += q.y; lx.z += q.z;
-    gs[0].x = fmaf(0.5f * s.x, q.x, gs[0].x); gs[0].y = fmaf(0.5f * s.y, q.y, gs[0].y);
-    gs[0].z = fmaf(0.5f * s.z, q.z, gs[0].z);
-    q = jt_times(J1, gs[0]);
-    scatter_step(gF, g, st, gs);
-    return make_float3(lx.x + q.x, lx.y + q.y, lx.z + q.z);
+    float3 p[4];
+    p[0] = x;
+    float fx, fy, fz;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        locate(C, f, g, p[k], fx, fy, fz);
+        const float3 v = trilerp(C.v, fx, fy, fz);
+        const float h = k == 2 ? 1.f : 0.5f;
+        p[k + 1] = make_float3(fmaf(h * s.x, v.x, x.x), fmaf(h * s.y, v.y, x.y), fmaf(h * s.z, v.z, x.z));
+    }
+    const float3 s6l = make_float3(s.x / 6.f * lm.x, s.y / 6.f * lm.y, s.z / 6.f * lm.z);
+    const float3 s3l = make_float3(s.x / 3.f * lm.x, s.y / 3.f * lm.y, s.z / 3.f * lm.z);
+    float3 lx = lm, w = s6l;   // w: the stage's g
+    float acc[8][3];
+    uint32_t acc_node = ~0u;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+        locate(C, f, g, p[k], fx, fy, fz);
+        if (C.node != acc_node) {
+            if (k < 3) add_cell(gF, g, acc_node, acc);
+            acc_node = C.node;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float wt = ((j & 1) ? fx : 1.f - fx) * ((j & 2) ? fy : 1.f - fy) * ((j & 4) ? fz : 1.f - fz);
+            acc[j][0] = fmaf(wt, w.x, acc[j][0]);
+            acc[j][1] = fmaf(wt, w.y, acc[j][1]);
+            acc[j][2] = fmaf(wt, w.z, acc[j][2]);
+        }
+        const float3 q = grad_dot(C, fx, fy, fz, w);
+        lx.x += q.x; lx.y += q.y; lx.z += q.z;
+        if (k > 0) {
+            const float h = k == 3 ? 1.f : 0.5f;
+            const float3 b = k == 1 ? s6l : s3l;
+            w = make_float3(fmaf(h * s.x, q.x, b.x), fmaf(h * s.y, q.y, b.y), fmaf(h * s.z, q.z, b.z));
+        }
+    }
+    add_cell(gF, g, acc_node, acc);
+    return lx;
 }
 
 // dk = J dp, column by column.
@@ -443,15 +464,23 @@ __global__ void tape_chain_kernel(const BlockDev *__restrict__ blk, int32_t L, i
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = perm[i];
         float3 l = make_float3(grad[3 * o + 0] * B.h[0], grad[3 * o + 1] * B.h[1], grad[3 * o + 2] * B.h[2]);
-        for (int32_t sg = last_segment(exitc[i], L, C); sg >= 0; --sg) {
-            float *m = mat + (size_t)sg * 9 * P + i;
-            float M[3][3];
+        int32_t sg = last_segment(exitc[i], L, C);
+        float *m = mat + (size_t)max(sg, 0) * 9 * P + i;
+        float M[9], N[9];   // N: the next segment's, loaded ahead of the stores
 #pragma unroll
-            for (int k = 0; k < 9; ++k) M[k / 3][k % 3] = m[(size_t)k * P];
+        for (int k = 0; k < 9; ++k) N[k] = sg >= 0 ? m[(size_t)k * P] : 0.f;
+        for (; sg >= 0; --sg, m -= (size_t)9 * P) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) M[k] = N[k];
+            if (sg > 0) {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) N[k] = *(m - (size_t)(9 - k) * P);
+            }
             m[0] = l.x;
             m[(size_t)P] = l.y;
             m[(size_t)2 * P] = l.z;
-            l = jt_times(M, l);
+            const float J[3][3] = {{M[0], M[1], M[2]}, {M[3], M[4], M[5]}, {M[6], M[7], M[8]}};
+            l = jt_times(J, l);
         }
         out[3 * o + 0] = l.x * B.inv_h[0];
         out[3 * o + 1] = l.y * B.inv_h[1];
@@ -536,13 +565,13 @@ __device__ double sym3_max_eig(const double C[3][3]) {
     if (p1 <= 1e-300 * (q * q + 1.0)) return fmax(C[0][0], fmax(C[1][1], C[2][2]));
     const double p2 = (C[0][0] - q) * (C[0][0] - q) + (C[1][1] - q) * (C[1][1] - q) +
                       (C[2][2] - q) * (C[2][2] - q) + 2.0 * p1;
-    const double p = sqrt(p2 / 6.0);
+    const double p = sqrt(p2 / 6.0), ip = 1.0 / p;   // one division: FP64 runs at 1/64 of the FP32 rate here
     double Bm[3][3];
     for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) Bm[a][b] = (C[a][b] - (a == b ? q : 0.0)) / p;
-    const double detB = Bm[0][0] * (Bm[1][1] * Bm[2][2] - Bm[1][2] * Bm[2][1]) -
-                        Bm[0][1] * (Bm[1][0] * Bm[2][2] - Bm[1][2] * Bm[2][0]) +
-                        Bm[0][2] * (Bm[1][0] * Bm[2][1] - Bm[1][1] * Bm[2][0]);
+        for (int b = a; b < 3; ++b) Bm[a][b] = (C[a][b] - (a == b ? q : 0.0)) * ip;
+    const double detB = Bm[0][0] * (Bm[1][1] * Bm[2][2] - Bm[1][2] * Bm[1][2]) -
+                        Bm[0][1] * (Bm[0][1] * Bm[2][2] - Bm[1][2] * Bm[0][2]) +
+                        Bm[0][2] * (Bm[0][1] * Bm[1][2] - Bm[1][1] * Bm[0][2]);
     const double r = fmin(1.0, fmax(-1.0, detB / 2.0));
     const double phi = acos(r) / 3.0;
     return q + 2.0 * p * cos(phi);
@@ -696,7 +725,8 @@ bto_status bto_tape_forward(bto_tape *t, const float *d_seeds, const void *const
     if (place) {
         const Bins bins = {{t->bsh[0], t->bsh[1], t->bsh[2]}, {t->bn[0], t->bn[1], t->bn[2]}};
         tape_bin_kernel<<<grid, 256, 0, s>>>(t->d_block, t->P, d_seeds, bins, t->bins, place);
-        tape_scan_kernel<<<1, 1024, 0, s>>>(t->bins, t->bins + kMaxBins, t->bn[0] * t->bn[1] * t->bn[2]);
+        tape_scan_kernel<<<1, 1024, 0, s>>>(reinterpret_cast<int4 *>(t->bins),
+                                            reinterpret_cast<int4 *>(t->bins + kMaxBins));
     }
     tape_init_kernel<<<grid, 256, 0, s>>>(t->d_block, t->P, d_seeds, t->bins + kMaxBins, place, t->ckpt, t->exitc,
                                           t->perm);

@@ -242,27 +242,6 @@ __device__ __forceinline__ int rk4_step(float3 &x, const void *__restrict__ fiel
     return rk4_step_src(x, GlobalSrc<LAYOUT>{field, g.nnx, g.nnxy, g.nodes, err}, g, s, q);
 }
 
-// Brings the node rows of the cell at x (a point of the closed box) of
-// another cycle's field into L2. A particle moves a fraction of a cell per
-// cycle, so these are mostly the rows its next step samples; nothing else
-// has read that field yet, and without this the first sample of every step
-// waits for DRAM.
-template <int LAYOUT>
-__device__ __forceinline__ void prefetch_cell(const void *__restrict__ field, const Geo &g, const float3 x) {
-    int i, j, k;
-    float f;
-    cell_coord(x.x, g.cmx, i, f);
-    cell_coord(x.y, g.cmy, j, f);
-    cell_coord(x.z, g.cmz, k, f);
-    const uint32_t node = (uint32_t)i + g.nnx * (uint32_t)j + g.nnxy * (uint32_t)k;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
-        const char *p = reinterpret_cast<const char *>(field) + (LAYOUT == LAYOUT_F4 ? 16ull : 12ull) * nd;
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-    }
-}
-
 // Termination location (the paper's future work, Sec. 6): the chord from the
 // last in-block position x to the first point q found outside is clipped to
 // the block, t = largest value in [0, 1] with x + t (q - x) inside; the exit

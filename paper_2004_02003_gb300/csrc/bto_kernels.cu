@@ -207,7 +207,6 @@ __global__ void __launch_bounds__(kRegionAlign) interval_kernel(const AdvectArgs
         if (c + 1 < cycles) {
             entry += a.nb;
             next = *entry;
-            if (alive) prefetch_cell<LAYOUT>(next, g, x);
         }
         if (alive) {
             float3 q;
