@@ -75,7 +75,7 @@ __device__ __forceinline__ int64_t orient(const LPt &a, const LPt &b, const LPt 
                 d.z - a.z);
 }
 
-__device__ __noinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e);
+__device__ __forceinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e);
 
 // Sign of the 5 x 5 determinant with rows (x, y, z, w, 1) of t0..t3, e
 // under the perturbed lifting: negative when e is inside the circumsphere of
@@ -108,27 +108,26 @@ __device__ __noinline__ int lifted_sign(const LPt (&t)[4], const LPt &e) {
     return perturbed_sign(t, e);
 }
 
-// The sign when the unperturbed determinant is zero: point k of
-// (t0, t1, t2, t3, e) carries the term (-1)^(k+3) * (-orient(the other
-// four, in order)); the lowest-ranked point with a non-zero term decides.
-__device__ __noinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e) {
-    const LPt *p[5] = {&t[0], &t[1], &t[2], &t[3], &e};
-    bool used[5] = {false, false, false, false, false};
-    for (int round = 0; round < 5; ++round) {
-        int k = -1;
-        for (int m = 0; m < 5; ++m)
-            if (!used[m] && (k < 0 || p[m]->rank < p[k]->rank)) k = m;
-        used[k] = true;
-        const LPt *q[4];
-        for (int m = 0, n = 0; m < 5; ++m)
-            if (m != k) q[n++] = p[m];
-        const int64_t o = -orient(*q[0], *q[1], *q[2], *q[3]);
+// The sign when the unperturbed determinant is zero: the lowest-ranked of the
+// five points with a non-zero cofactor decides. e's own cofactor is orient(T)
+// > 0 (outside); vertex k's is -orient(T with e in its place), e's weight at
+// that vertex, so a vertex that e has a positive weight at makes e inside.
+__device__ __forceinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e) {
+    int64_t rank = e.rank;
+    int sign = 1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (t[k].rank >= rank) continue;
+        LPt u[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) u[m] = m == k ? e : t[m];
+        const int64_t o = orient(u[0], u[1], u[2], u[3]);
         if (o != 0) {
-            const int64_t c = ((k + 3) & 1) ? -o : o;
-            return c > 0 ? 1 : -1;
+            rank = t[k].rank;
+            sign = o > 0 ? -1 : 1;
         }
     }
-    return 0;
+    return sign;
 }
 
 __device__ __forceinline__ int64_t lattice_rank(int3 S, int64_t x, int64_t y, int64_t z) {
@@ -227,6 +226,26 @@ __device__ bool sphere_fits(const double (&ctr)[3], double r2, int3 S, int64_t c
     return true;
 }
 
+// sphere_fits from the FP32 sphere: 1 or 0 where every compared distance is
+// clear of its plane by 1e-4 (r + 1) (the FP32 centre and radius are within
+// 1e-6 (r + 1) of the exact ones), -1 when one is closer.
+__device__ __forceinline__ int fits_clearly(const float (&ctr)[3], float r2, int3 S, int cx, int cy, int cz, int64_t x0,
+                                            int64_t x1, int64_t y0, int64_t y1, int64_t z0, int64_t z1) {
+    const float rad = sqrtf(r2), tol = 1e-4f * (rad + 1.f);
+    const float lo[3] = {(float)(x0 - cx) - 1.f, (float)(y0 - cy) - 1.f, (float)(z0 - cz) - 1.f};
+    const float hi[3] = {(float)(x1 - cx) + 1.f, (float)(y1 - cy) + 1.f, (float)(z1 - cz) + 1.f};
+    const bool open_lo[3] = {x0 > 0, y0 > 0, z0 > 0};
+    const bool open_hi[3] = {x1 < S.x - 1, y1 < S.y - 1, z1 < S.z - 1};
+    int fit = 1;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const float a = ctr[m] - rad - lo[m], b = hi[m] - ctr[m] - rad;   // room below and above
+        if ((open_lo[m] && a < -tol) || (open_hi[m] && b < -tol)) return 0;
+        if ((open_lo[m] && !(a > tol)) || (open_hi[m] && !(b > tol))) fit = -1;
+    }
+    return fit;
+}
+
 // Every routine from here on is warp-cooperative: the 32 lanes of a warp
 // solve one missing entry together. They hold the same simplex, split the
 // window's points between them (point k of the window goes to lane k mod
@@ -310,6 +329,11 @@ __device__ __forceinline__ void rank_coords(int3 S, int64_t r, int64_t (&p)[3]) 
     const int q = rr / S.x;
     p[1] = q % S.y;
     p[2] = q / S.y;
+}
+
+__device__ __forceinline__ unsigned gcd(unsigned a, unsigned b) {
+    while (b) { const unsigned r = a % b; a = b; b = r; }
+    return a;
 }
 
 // The walk ended with one starting point (vertex kf of T) at weight exactly
@@ -399,9 +423,19 @@ __device__ __noinline__ bool across_facet(int3 S, const uint8_t *__restrict__ va
         const int64_t rows = (int64_t)S.y * S.z, budget = kHullScanWork / 32;
         int64_t work = 0;
         bool stop = false;                          // a far-side valid point, or out of budget
-        for (int64_t row = lane; row < rows && !stop; row += 32) {
+        // Each lane keeps the rows lane, lane + 32, ...; it takes them in the
+        // order of multiples of a number coprime to their count, and the warp
+        // ends as soon as one lane has stopped: a valid point on the far side
+        // is mostly met within a few rows spread over the lattice.
+        const unsigned per = (unsigned)((rows + 31) / 32);
+        unsigned hop = per * 5 / 8 + 1;
+        while (gcd(hop, per) != 1) ++hop;
+        unsigned at = 0;
+        for (unsigned k = 0; k < per && !__any_sync(kAll, stop); ++k, at = (at + hop) % per) {
+            const int64_t row = lane + 32ll * at;
+            if (row >= rows) continue;
             const int64_t y = (int)row % S.y, z = (int)row / S.y;
-            if (++work > budget) { stop = true; break; }
+            if (++work > budget) { stop = true; continue; }
             int64_t t0, t1;
             if (!positive_range(sg * nx, sg * (ny * (y - cy) + nz * (z - cz) + d), -cx, (int64_t)S.x - 1 - cx, t0, t1))
                 continue;
@@ -484,8 +518,7 @@ __device__ __forceinline__ bool inside_sphere(const Sphere &S, const LPt (&T)[4]
                                 S.m[2] * (uint64_t)(int64_t)p.z + S.k);
     if (F != 0) return F < 0;
     if (T[0].rank == p.rank || T[1].rank == p.rank || T[2].rank == p.rank || T[3].rank == p.rank) return false;
-    const LPt t4[4] = {T[0], T[1], T[2], T[3]};   // the copy keeps T itself in registers
-    return perturbed_sign(t4, p) < 0;
+    return perturbed_sign(T, p) < 0;
 }
 
 // The valid points around a tile of kTileX x kTileY x kTileZ entries, one
@@ -517,6 +550,7 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
     const int side = 2 * R + 1, rows = side * side;
     const uint32_t wmask = ((1u << side) - 1u) << (kMaxWindow - R);
     const uint32_t ends = (1u << (kMaxWindow - R)) | (1u << (kMaxWindow + R));
+    const unsigned inv_side = 65536u / (unsigned)side + 1u;   // row / side for rows < 2^16 / side
     for (int it = 0; it < kMaxPivots; ++it) {
         // entering point: among the valid window points inside the
         // circumsphere of T, the deepest (later the lowest-ranked) one. A
@@ -535,12 +569,12 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
         int64_t best = kNone;
         unsigned bhi = 0, blo = 0;   // the lane's best depth key (depth_key), 0: none
         for (int row = lane; row < rows; row += 32) {
-            const int rz = row / side, dy = row - rz * side - R, dz = rz - R;
+            const int rz = (int)(((unsigned)row * inv_side) >> 16), dy = row - rz * side - R, dz = rz - R;
             uint32_t m = (win[dy + kRowsY * dz] >> lx) & wmask;
             if (shell && dy > -R && dy < R && dz > -R && dz < R) m &= ends;
             if (!m) continue;
             const float fy = (float)dy - fc1, fz = (float)dz - fc2;
-            const int64_t r0 = lattice_rank(S, (int64_t)cx - kMaxWindow, (int64_t)cy + dy, (int64_t)cz + dz);
+            const int r0 = cx - kMaxWindow + S.x * (cy + dy + S.y * (cz + dz));   // the row's ranks are r0 + bit, below 2^31
             if (deep) {
 #pragma unroll
                 for (int dir = 0; dir < 2; ++dir) {
@@ -552,7 +586,7 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
                         const float fx = (float)dx - fc0;
                         const float d2 = fx * fx + fy * fy + fz * fz;
                         if (d2 > fr2) break;
-                        const int64_t r = r0 + bit;
+                        const int r = r0 + bit;
                         const unsigned long long key = depth_key(sp.r2 - d2, r);
                         const unsigned khi = (unsigned)(key >> 32), klo = (unsigned)key;
                         if (khi < bhi) break;
@@ -584,71 +618,88 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
         } else {
             best = warp_min(best);
         }
-        // orientations with vertex k replaced, one vertex to a lane: by q
-        // (oq) and, when a point enters, by that point (oe)
+        // orientations with vertex k replaced, one vertex to a lane (lanes
+        // 4 apart hold the same): by q (oq) and, when a point enters, by
+        // that point (oe)
         const LPt q0 = {0, 0, 0, -1};
         const int mine = lane & 3;
-        const int64_t o = sp.d;
         LPt u[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) u[k] = mine == k ? q0 : T[k];
-        const int64_t oq_mine = orient(u[0], u[1], u[2], u[3]);
+        const int64_t oq = orient(u[0], u[1], u[2], u[3]);
+        const int64_t rank_mine = mine == 0 ? T[0].rank : (mine == 1 ? T[1].rank : (mine == 2 ? T[2].rank : T[3].rank));
         if (best == kNone) {
             settled = true;
+            const unsigned far = __ballot_sync(kAll, rank_mine >= P) & 15u;
+            const unsigned zero = __ballot_sync(kAll, oq == 0) & 15u;
+            if (far == 0) {
+                // the circumsphere must fit in the window: then no lattice
+                // point outside the window is inside it. FP32 decides when
+                // the sphere ends clearly on one side of every plane; FP64
+                // otherwise.
+                const int fit = fits_clearly(sp.c, sp.r2, S, cx, cy, cz, x0, x1, y0, y1, z0, z1);
+                if (fit == 0) return 0;
+                if (fit < 0) {
+                    const LPt t4[4] = {T[0], T[1], T[2], T[3]};   // the copy keeps T itself in registers
+                    double ctr[3], r2;
+                    circumsphere(t4, ctr, r2);
+                    if (!sphere_fits(ctr, r2, S, cx, cy, cz, x0, x1, y0, y1, z0, z1)) return 0;
+                }
+            } else if ((far & (far - 1)) != 0 || (far & ~zero) != 0) {
+                // a starting point with weight above 0: q is outside the
+                // hull of the window's valid points
+                return 0;
+            }
             // optimal: q's barycentric coordinates in T
-            int64_t ol[4];
-            int nfar = 0, kf = -1;
-            int64_t ofar = 0;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                ol[k] = __shfl_sync(kAll, (long long)oq_mine, k);
-                lam[k] = (double)ol[k] / (double)o;
-                if (T[k].rank >= P) { ++nfar; kf = k; ofar = ol[k]; }
-            }
-            // the circumsphere (FP64) must fit in the window: then no
-            // lattice point outside the window is inside it
-            if (nfar == 0) {
-                const LPt t4[4] = {T[0], T[1], T[2], T[3]};
-                double ctr[3], r2;
-                circumsphere(t4, ctr, r2);
-                return sphere_fits(ctr, r2, S, cx, cy, cz, x0, x1, y0, y1, z0, z1) ? 1 : 0;
-            }
-            // a starting point with weight above 0: q is outside the hull
-            // of the window's valid points; with weight 0: q is on a facet
-            if (nfar > 1 || ofar != 0) return 0;
+            for (int k = 0; k < 4; ++k) lam[k] = (double)__shfl_sync(kAll, (long long)oq, k) / (double)sp.d;
+            if (far == 0) return 1;
+            // a starting point with weight 0: q is on a facet
             LPt t4[4] = {T[0], T[1], T[2], T[3]};
-            if (!across_facet(S, valid, cx, cy, cz, x0, x1, y0, y1, z0, z1, t4, kf)) return 0;
+            if (!across_facet(S, valid, cx, cy, cz, x0, x1, y0, y1, z0, z1, t4, __ffs(far) - 1)) return 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) T[k] = t4[k];
             return 1;
         }
         settled = false;
-        int64_t bc[3];
-        rank_coords(S, best, bc);
-        const LPt e = {(int32_t)(bc[0] - cx), (int32_t)(bc[1] - cy), (int32_t)(bc[2] - cz), best};
+        const unsigned b32 = (unsigned)best;
+        const int ez = (int)(b32 / (unsigned)(S.x * S.y)), ey = (int)(b32 / (unsigned)S.x) - ez * S.y;
+        const LPt e = {(int32_t)(b32 % (unsigned)S.x) - cx, ey - cy, ez - cz, best};
 #pragma unroll
         for (int k = 0; k < 4; ++k) u[k] = mine == k ? e : T[k];
-        const int64_t oe_mine = orient(u[0], u[1], u[2], u[3]);
-        // ratio test: leaving vertex k minimises lambda_k / d_k over d_k > 0,
-        // with lambda_k = O_k(q) / O and d_k = O_k(e) / O (O_k: orientation
-        // with vertex k replaced); ties go to the lowest rank
-        int leave = -1;
-        int64_t bq = 0, be = 0, brank = 0;
+        const int64_t oe = orient(u[0], u[1], u[2], u[3]);
+        // ratio test: leaving vertex k minimises lambda_k / d_k = oq / oe
+        // over oe > 0 (orient(T) > 0 divides out); ties go to the lowest
+        // rank. FP32 quotients (three roundings, 2e-7 relative) single out
+        // the vertex unless another is within 1e-5 of the least; exact zeros
+        // tie among themselves; other near ties are compared exactly.
+        const float ratio = oe > 0 ? (float)oq / (float)oe : INFINITY;
+        float least = fminf(ratio, __shfl_xor_sync(kAll, ratio, 1));
+        least = fminf(least, __shfl_xor_sync(kAll, least, 2));
+        if (least == INFINITY) return 0;   // cannot happen for a point inside the circumsphere
+        const unsigned near = __ballot_sync(kAll, ratio <= least * 1.00001f) & 15u;
+        int leave = __ffs(near) - 1;
+        if (near & (near - 1)) {
+            int64_t bq = 0, be = 0, brank = 0;
+            leave = -1;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t oe = __shfl_sync(kAll, (long long)oe_mine, k);
-            const int64_t oq = __shfl_sync(kAll, (long long)oq_mine, k);
-            if (oe <= 0) continue;   // o > 0: d_k has oe's sign
-            // compare oq / oe against bq / be (both denominators positive)
-            bool better = leave < 0;
-            if (!better) {
-                const i128 lhs = (i128)oq * be, rhs = (i128)bq * oe;
-                better = lhs < rhs || (lhs == rhs && T[k].rank < brank);
+            for (int k = 0; k < 4; ++k) {
+                if (!(near >> k & 1u)) continue;
+                const int64_t kq = __shfl_sync(kAll, (long long)oq, k), ke = __shfl_sync(kAll, (long long)oe, k);
+                bool better = leave < 0;
+                if (!better) {
+                    // compare kq / ke against bq / be (both denominators positive)
+                    if (least == 0.f) {
+                        better = T[k].rank < brank;
+                    } else {
+                        const i128 lhs = (i128)kq * be, rhs = (i128)bq * ke;
+                        better = lhs < rhs || (lhs == rhs && T[k].rank < brank);
+                    }
+                }
+                if (better) { leave = k; bq = kq; be = ke; brank = T[k].rank; }
             }
-            if (better) { leave = k; bq = oq; be = oe; brank = T[k].rank; }
         }
-        if (leave < 0) return 0;   // cannot happen for a point inside the circumsphere
-        // the new orientation is be > 0: T stays positively oriented
+        // the new orientation is the leaving vertex's oe > 0: T stays positively oriented
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k == leave) T[k] = e;
@@ -659,25 +710,25 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
 // ---- Faces: the same program in a face's two free coordinates ----------
 
 struct LPt2 {
-    int64_t u, v;      // free coordinates relative to the query point
+    int32_t u, v;      // free coordinates relative to the query point
     int64_t rank;
 };
 
 // Counter-clockwise orientation of (a, b, c): positive when counter-clockwise.
 // Coordinates differ by less than 2^12 (as for LPt), so 64 bits are exact.
 __device__ __forceinline__ int64_t orient2(const LPt2 &a, const LPt2 &b, const LPt2 &c) {
-    return (b.u - a.u) * (c.v - a.v) - (b.v - a.v) * (c.u - a.u);
+    return (int64_t)(b.u - a.u) * (c.v - a.v) - (int64_t)(b.v - a.v) * (c.u - a.u);
 }
 
-__device__ __noinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e);
+__device__ __forceinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e);
 
 // Sign of the 4 x 4 determinant with rows (u, v, w, 1) of t0, t1, t2, e under
 // the perturbed lifting w = u^2 + v^2 + d_rank: positive when e is inside the
 // circumcircle of the counter-clockwise triangle (t0, t1, t2). Translated so
 // that e is the origin, the unperturbed part is the 3 x 3 determinant of the
 // rows (p - e, |p - e|^2).
-__device__ __noinline__ int lifted_sign2(const LPt2 (&t)[3], const LPt2 &e) {
-    int64_t r[3][3];
+__device__ __forceinline__ int lifted_sign2(const LPt2 (&t)[3], const LPt2 &e) {
+    int32_t r[3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         r[i][0] = t[i].u - e.u;
@@ -689,27 +740,24 @@ __device__ __noinline__ int lifted_sign2(const LPt2 (&t)[3], const LPt2 &e) {
     return perturbed_sign2(t, e);
 }
 
-// The sign when the unperturbed determinant is zero: the lifted entry of
-// point k of (t0, t1, t2, e) has the cofactor (-1)^k orient2(the other three,
-// in order); the lowest-ranked point with a non-zero cofactor decides.
-__device__ __noinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e) {
-    const LPt2 *p[4] = {&t[0], &t[1], &t[2], &e};
-    bool used[4] = {false, false, false, false};
-    for (int round = 0; round < 4; ++round) {
-        int k = -1;
-        for (int m = 0; m < 4; ++m)
-            if (!used[m] && (k < 0 || p[m]->rank < p[k]->rank)) k = m;
-        used[k] = true;
-        const LPt2 *q[3];
-        for (int m = 0, n = 0; m < 4; ++m)
-            if (m != k) q[n++] = p[m];
-        const int64_t o = orient2(*q[0], *q[1], *q[2]);
+// The sign when the unperturbed determinant is zero, as perturbed_sign: e's
+// own cofactor says outside, vertex k's has the sign of e's weight there.
+__device__ __forceinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e) {
+    int64_t rank = e.rank;
+    int sign = -1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (t[k].rank >= rank) continue;
+        LPt2 u[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) u[m] = m == k ? e : t[m];
+        const int64_t o = orient2(u[0], u[1], u[2]);
         if (o != 0) {
-            const int64_t c = (k & 1) ? -o : o;
-            return c > 0 ? 1 : -1;
+            rank = t[k].rank;
+            sign = o > 0 ? 1 : -1;
         }
     }
-    return 0;
+    return sign;
 }
 
 // Circumcircle of T (centre and squared radius, FP64), for the filter.
@@ -727,7 +775,7 @@ __device__ __noinline__ void circumcircle(const LPt2 (&T)[3], double (&ctr)[2], 
 // The circumcircle of T for the face walk's filter, as circumsphere_f:
 // exact 64-bit Cramer numerators, FP32 quotients.
 __device__ __forceinline__ void circumcircle_f(const LPt2 (&T)[3], float (&c)[2], float &r2) {
-    const int64_t bx = T[1].u - T[0].u, by = T[1].v - T[0].v, cx = T[2].u - T[0].u, cy = T[2].v - T[0].v;
+    const int64_t bx = T[1].u - T[0].u, by = T[1].v - T[0].v, cx = T[2].u - T[0].u, cy = T[2].v - T[0].v;   // below 2^12
     const int64_t b2 = bx * bx + by * by, c2 = cx * cx + cy * cy;
     const float d = (float)(2 * (bx * cy - by * cx));
     const float ux = (float)(cy * b2 - by * c2) / d, uy = (float)(bx * c2 - cx * b2) / d;
@@ -738,7 +786,7 @@ __device__ __forceinline__ void circumcircle_f(const LPt2 (&T)[3], float (&c)[2]
 
 // Sets T to three far starting points around q (counter-clockwise).
 __device__ void start_triangle(int64_t P, LPt2 (&T)[3]) {
-    const int64_t far[3][2] = {{kFar, 0}, {-kFar, kFar}, {-kFar, -kFar}};
+    const int32_t far[3][2] = {{kFar, 0}, {-kFar, kFar}, {-kFar, -kFar}};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         T[k].u = far[k][0]; T[k].v = far[k][1];
@@ -785,7 +833,7 @@ __device__ __noinline__ bool across_edge(int3 S, const uint8_t *__restrict__ val
         pc[b] = v0 + w.y;
         const int64_t r = lattice_rank(S, pc[0], pc[1], pc[2]);
         if (!valid[r] || r == A.rank || r == B.rank) continue;
-        const LPt2 p = {pc[a] - c[a], pc[b] - c[b], r};
+        const LPt2 p = {(int32_t)(pc[a] - c[a]), (int32_t)(pc[b] - c[b]), r};
         const int64_t so = orient2(A, B, p);
         if (so == 0) continue;
         if ((so > 0) == (sf > 0)) { far_pt = true; continue; }
@@ -817,7 +865,7 @@ __device__ __noinline__ bool across_edge(int3 S, const uint8_t *__restrict__ val
             pc[b] = v0 + w.y;
             const int64_t r = lattice_rank(S, pc[0], pc[1], pc[2]);
             if (!valid[r] || r == A.rank || r == B.rank || r == D.rank) continue;
-            const LPt2 p = {pc[a] - c[a], pc[b] - c[b], r};
+            const LPt2 p = {(int32_t)(pc[a] - c[a]), (int32_t)(pc[b] - c[b]), r};
             inside = lifted_sign2(t3, p) > 0;
         }
         inside = __any_sync(kAll, inside);
@@ -857,38 +905,57 @@ __device__ __noinline__ bool across_edge(int3 S, const uint8_t *__restrict__ val
     return false;
 }
 
+// circle_fits from the FP32 circle, as fits_clearly.
+__device__ __forceinline__ int circle_fits_clearly(const float (&ctr)[2], float r2, int lo_u, int hi_u, int lo_v,
+                                                   int hi_v, bool open_lu, bool open_hu, bool open_lv, bool open_hv) {
+    const float rad = sqrtf(r2), tol = 1e-4f * (rad + 1.f);
+    const float room[4] = {ctr[0] - rad - (float)lo_u + 1.f, (float)hi_u + 1.f - ctr[0] - rad,
+                           ctr[1] - rad - (float)lo_v + 1.f, (float)hi_v + 1.f - ctr[1] - rad};
+    const bool open[4] = {open_lu, open_hu, open_lv, open_hv};
+    int fit = 1;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        if (open[m] && room[m] < -tol) return 0;
+        if (open[m] && !(room[m] > tol)) fit = -1;
+    }
+    return fit;
+}
+
 // The walk of `walk` on the face through c whose free axes are a < b: the
 // window is the square of radius R around c on that face, its points in
-// rank order (axis a fastest). Returns 1 with the triangle and q's
-// barycentric coordinates, or 0.
-__device__ __noinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], int a, int b, int R,
-                     LPt2 (&T)[3], double (&lam)[3]) {
+// rank order (axis a fastest), shared out point by point. Returns 1 with the
+// triangle and q's barycentric coordinates, or 0.
+__device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], int a, int b,
+                                     int R, bool &settled, LPt2 (&T)[3], double (&lam)[3]) {
     const int lane = threadIdx.x & 31;
     const int64_t P = (int64_t)S.x * S.y * S.z;
-    const int64_t ext[3] = {S.x, S.y, S.z};
     const LPt2 q0 = {0, 0, -1};
-    const int64_t u0 = max(c[a] - R, (int64_t)0), u1 = min(c[a] + R, ext[a] - 1);
-    const int64_t v0 = max(c[b] - R, (int64_t)0), v1 = min(c[b] + R, ext[b] - 1);
-    const int wu = (int)(u1 - u0 + 1), W = wu * (int)(v1 - v0 + 1);
+    // a is 0 or 1, b is 1 or 2
+    const int ca = (int)(a == 0 ? c[0] : c[1]), cb = (int)(b == 1 ? c[1] : c[2]);
+    const int ea = a == 0 ? S.x : S.y, eb = b == 1 ? S.y : S.z;
+    const int sa = a == 0 ? 1 : S.x, sb = b == 1 ? S.x : S.x * S.y;   // rank steps of the free axes
+    const int rq = (int)lattice_rank(S, c[0], c[1], c[2]);
+    const int u0 = max(ca - R, 0), u1 = min(ca + R, ea - 1), v0 = max(cb - R, 0), v1 = min(cb + R, eb - 1);
+    const int wu = u1 - u0 + 1, W = wu * (v1 - v0 + 1);
     for (int it = 0; it < kMaxPivots; ++it) {
         float fc[2], fr2e;
         circumcircle_f(T, fc, fr2e);
         const float fc0 = fc[0], fc1 = fc[1];
         const float fr2 = fr2e * (1.0f + 1e-4f) + 1e-2f;   // as in walk
         const bool deep = it < kDeepPivots;   // the pivot rule of walk
+        const bool shell = settled && it == 0;
         int64_t best = kNone;
         unsigned long long bkey = 0;
         for (WinIter w(wu, 1 << 30, lane); w.k < W; w.step()) {
-            int64_t pc[3] = {c[0], c[1], c[2]};
-            pc[a] = u0 + w.x;
-            pc[b] = v0 + w.y;
-            const int64_t r = lattice_rank(S, pc[0], pc[1], pc[2]);
+            const int du = u0 + w.x - ca, dv = v0 + w.y - cb;
+            if (shell && max(abs(du), abs(dv)) < R) continue;
+            const int r = rq + du * sa + dv * sb;
             if (!valid[r]) continue;
-            const float du = (float)(pc[a] - c[a]) - fc0, dv = (float)(pc[b] - c[b]) - fc1;
-            const float d2 = du * du + dv * dv;
+            const float fu = (float)du - fc0, fv = (float)dv - fc1;
+            const float d2 = fu * fu + fv * fv;
             if (d2 > fr2) continue;
             if (T[0].rank == r || T[1].rank == r || T[2].rank == r) continue;
-            const LPt2 cand = {pc[a] - c[a], pc[b] - c[b], r};
+            const LPt2 cand = {du, dv, r};
             if (deep) {
                 const unsigned long long key = depth_key(fr2e - d2, r);
                 if (key > bkey && lifted_sign2(T, cand) > 0) bkey = key;
@@ -905,29 +972,44 @@ __device__ __noinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, con
         }
         const int64_t o = orient2(T[0], T[1], T[2]);   // > 0: T is kept counter-clockwise
         if (best == kNone) {
-            int64_t ol[3];
+            settled = true;
+            int64_t ol[3], ofar = 0;
             int nfar = 0, kf = -1;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 LPt2 u[3] = {T[0], T[1], T[2]};
                 u[k] = q0;
                 ol[k] = orient2(u[0], u[1], u[2]);
-                lam[k] = (double)ol[k] / (double)o;
-                if (T[k].rank >= P) { ++nfar; kf = k; }
+                if (T[k].rank >= P) { ++nfar; kf = k; ofar = ol[k]; }
             }
+            const LPt2 t3[3] = {T[0], T[1], T[2]};   // the copies keep T itself in registers
             if (nfar == 0) {
-                double ctr[2], r2;
-                circumcircle(T, ctr, r2);
-                return circle_fits(ctr, r2, S, c, a, b, u0, u1, v0, v1) ? 1 : 0;
+                const int fit = circle_fits_clearly(fc, fr2e, u0 - ca, u1 - ca, v0 - cb, v1 - cb, u0 > 0, u1 < ea - 1,
+                                                    v0 > 0, v1 < eb - 1);
+                if (fit == 0) return 0;
+                if (fit < 0) {
+                    double ctr[2], r2;
+                    circumcircle(t3, ctr, r2);
+                    if (!circle_fits(ctr, r2, S, c, a, b, u0, u1, v0, v1)) return 0;
+                }
+            } else if (nfar > 1 || ofar != 0) {
+                return 0;
             }
-            if (nfar > 1 || ol[kf] != 0) return 0;
-            return across_edge(S, valid, c, a, b, u0, u1, v0, v1, T, kf) ? 1 : 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) lam[k] = (double)ol[k] / (double)o;
+            if (nfar == 0) return 1;
+            LPt2 x3[3] = {T[0], T[1], T[2]};
+            if (!across_edge(S, valid, c, a, b, u0, u1, v0, v1, x3, kf)) return 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) T[k] = x3[k];
+            return 1;
         }
+        settled = false;
         int64_t bc[3];
         rank_coords(S, best, bc);
-        const LPt2 e = {bc[a] - c[a], bc[b] - c[b], best};
+        const LPt2 e = {(int32_t)(a == 0 ? bc[0] : bc[1]) - ca, (int32_t)(b == 1 ? bc[1] : bc[2]) - cb, best};
         int leave = -1;
-        int64_t bq = 0, be = 0;
+        int64_t bq = 0, be = 0, brank = 0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             LPt2 u[3] = {T[0], T[1], T[2]};
@@ -939,13 +1021,15 @@ __device__ __noinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, con
             bool better = leave < 0;
             if (!better) {
                 const int64_t lhs = oq * be, rhs = bq * oe;   // below 2^50
-                better = lhs < rhs || (lhs == rhs && T[k].rank < T[leave].rank);
+                better = lhs < rhs || (lhs == rhs && T[k].rank < brank);
             }
-            if (better) { leave = k; bq = oq; be = oe; }
+            if (better) { leave = k; bq = oq; be = oe; brank = T[k].rank; }
         }
         if (leave < 0) return 0;
-        T[leave] = e;
-        if (orient2(T[0], T[1], T[2]) < 0) { const LPt2 s = T[0]; T[0] = T[1]; T[1] = s; }
+        // the new orientation is be > 0: T stays counter-clockwise
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k == leave) T[k] = e;
     }
     return 0;
 }
@@ -1016,8 +1100,9 @@ constexpr int kTileN = kTileX * kTileY * kTileZ;
 // tiles than CTAs fit on the chip, and the hardware hands them out, so the
 // tiles inside a missing slab (256 entries) and those with none even out.
 // Bound by dependent integer chains of the pivots. A 128^3 lattice with
-// 137,210 missing entries (88,000 of them here): 61 -> 19 ms for the whole
-// fill against byte-wise window scans, one 32-entry chunk to a warp.
+// 137,210 missing entries (88,000 of them here), the whole fill: 61 ms with
+// byte-wise window scans and one 32-entry chunk to a warp, 20 ms with the row
+// words, 12 ms with the pivots' determinants and ratio test shared out too.
 __global__ void __launch_bounds__(kFillThreads) fill_interior_kernel(int3 S, int tx, int ty,
                                                                      const float *__restrict__ ends,
                                                                      const uint8_t *__restrict__ valid,
@@ -1137,7 +1222,8 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, con
             LPt2 T2[3];
             double l2[3];
             start_triangle(P, T2);
-            for (int R = 2; R <= kMaxWindow2 && !ok; ++R) ok = walk2(S, valid, c, a, b, R, T2, l2);
+            bool settled = false;
+            for (int R = 2; R <= kMaxWindow2 && !ok; ++R) ok = walk2(S, valid, c, a, b, R, settled, T2, l2);
             for (int k = 0; k < 3; ++k) { vtx[k] = T2[k].rank; lam[k] = l2[k]; }
             nv = 3;
         } else if (!flat && nfix == 2) {
