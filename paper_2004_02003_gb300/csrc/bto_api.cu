@@ -1047,11 +1047,7 @@ bto_status bto_fill_lattice(const int32_t lattice[3], const float *d_ends, const
         return BTO_ERR_INVALID_ARG;
     const int64_t P = (int64_t)lattice[0] * lattice[1] * lattice[2];
     if (P > (1ll << 31) - 1) return BTO_ERR_INVALID_ARG;
-    int dev = 0, sms = 0;
-    BTO_CUDA(cudaGetDevice(&dev));
-    BTO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((P + 255) / 256, (int64_t)sms * 8));
-    BTO_CUDA(bto::launch_fill_lattice(lattice, d_ends, d_valid, d_out, d_status, grid, (cudaStream_t)stream));
+    BTO_CUDA(bto::launch_fill_lattice(lattice, d_ends, d_valid, d_out, d_status, (cudaStream_t)stream));
     return BTO_OK;
 }
 

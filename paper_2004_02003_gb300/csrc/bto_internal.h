@@ -262,7 +262,7 @@ cudaError_t launch_stitch(const int32_t S[3], const float origin[3], const float
 cudaError_t launch_fill_delaunay(const int32_t S[3], const float *ends, const uint8_t *valid, float *out,
                                  uint8_t *status, cudaStream_t s);
 cudaError_t launch_fill_lattice(const int32_t S[3], const float *ends, const uint8_t *valid, float *out,
-                                uint8_t *status, int grid, cudaStream_t s);
+                                uint8_t *status, cudaStream_t s);
 cudaError_t launch_write_term(const BlockDev *blocks, int32_t nb, int64_t P, float4 *term,
                               float *seeds, float *ends, uint8_t *valid, int32_t *exit_cycle,
                               int grid, cudaStream_t s, const float4 *clip = nullptr,
