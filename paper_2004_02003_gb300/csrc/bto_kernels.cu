@@ -174,8 +174,12 @@ __global__ void __launch_bounds__(NT, MINB) advect_kernel(const AdvectArgs a) {
 // dependent samples, 2 warps per SM), 96 blocks of 16 to 96 cells with 7.5M
 // seeds over 32 cycles 5.15 -> 3.95 ms (bound by the L1 load path).
 // ---------------------------------------------------------------------------
+// Eight CTAs of 128 per SM (64 registers, 32 bytes spilled): 3.76 ms on the
+// 96 blocks against 3.92 at the compiler's own 72 registers, 4.80 at nine.
+constexpr int kIntervalCtas = 8;
+
 template <int LAYOUT>
-__global__ void __launch_bounds__(kRegionAlign) interval_kernel(const AdvectArgs a, const int32_t cycles,
+__global__ void __launch_bounds__(kRegionAlign, kIntervalCtas) interval_kernel(const AdvectArgs a, const int32_t cycles,
                                                                 const int group) {
     static_assert(kRegionAlign == 4 * kUnit, "a CTA is four units");
     __shared__ int kept[4];
