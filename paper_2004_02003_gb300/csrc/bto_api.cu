@@ -798,17 +798,17 @@ bto_status bto_end_interval_ex(bto_ctx *ctx, float *d_seeds, float *d_ends, uint
     if (ctx->cycle != ctx->L) return BTO_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
     const int L = ctx->L;
-    const int grid = aux_grid(ctx);
-    if (ctx->tiled)
-        BTO_CUDA(bto::launch_write_live_tiled(ctx->blocks, ctx->nb, ctx->tiles, ctx->unit_tile, ctx->tact[L & 1],
-                                              tile_counts(ctx, L), d_ends, d_valid, d_exit_cycle,
-                                              tiled_aux_grid(ctx), s));
-    else
-        BTO_CUDA(bto::launch_write_live(ctx->blocks, ctx->gblock, part_list(ctx),
-                                        ctx->slots, group_size(ctx), d_ends, d_valid, d_exit_cycle,
-                                        grid, s, ctx->derr));
-    BTO_CUDA(bto::launch_write_term(ctx->blocks, ctx->nb, ctx->P, ctx->term, d_seeds, d_ends,
-                                    d_valid, d_exit_cycle, grid, s, ctx->clip, d_exit_pos, d_exit_time));
+    if (!ctx->tiled) {
+        BTO_CUDA(bto::launch_end_interval(ctx->blocks, ctx->gblock, ctx->perm, ctx->slots, group_size(ctx),
+                                          part_list(ctx), ctx->term, ctx->clip, d_seeds, d_ends, d_valid, d_exit_cycle,
+                                          d_exit_pos, d_exit_time, ctx->derr, s));
+        ctx->cycle = 0;
+        return BTO_OK;
+    }
+    BTO_CUDA(bto::launch_write_live_tiled(ctx->blocks, ctx->nb, ctx->tiles, ctx->unit_tile, ctx->tact[L & 1],
+                                          tile_counts(ctx, L), d_ends, d_valid, d_exit_cycle, tiled_aux_grid(ctx), s));
+    BTO_CUDA(bto::launch_write_term(ctx->blocks, ctx->nb, ctx->P, ctx->term, d_seeds, d_ends, d_valid, d_exit_cycle,
+                                    aux_grid(ctx), s, ctx->clip, d_exit_pos, d_exit_time));
     return seed(ctx, s);
 }
 

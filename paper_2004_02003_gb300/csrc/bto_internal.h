@@ -249,6 +249,10 @@ cudaError_t launch_count_live_tiled(const BlockDev *blocks, int32_t nb, const Ti
 
 cudaError_t launch_seed(const BlockDev *blocks, const int32_t *gblock, const int32_t *perm,
                         int64_t slots, int group, PartList p, int grid, cudaStream_t s);
+cudaError_t launch_end_interval(const BlockDev *blocks, const int32_t *gblock, const int32_t *perm, int64_t slots,
+                                int group, PartList p, float4 *term, const float4 *clip, float *seeds, float *ends,
+                                uint8_t *valid, int32_t *exit_cycle, float *exit_pos, float *exit_time, int32_t *err,
+                                cudaStream_t s);
 cudaError_t launch_write_live(const BlockDev *blocks, const int32_t *gblock, PartList p, int64_t slots,
                               int group, float *ends, uint8_t *valid, int32_t *exit_cycle, int grid,
                               cudaStream_t s, int32_t *err = nullptr);

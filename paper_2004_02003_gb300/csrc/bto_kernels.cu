@@ -8,8 +8,10 @@
 //                         particles occupy no thread in later cycles
 //                         (Sec. 3.1, particle management)
 //   K3i interval_kernel   all cycles of an interval, fields resident
-//   K4 write_live_kernel  basis flows of surviving particles (Sec. 2.3)
-//      write_term_kernel  seeds and basis flows of terminated particles
+//   K4 end_interval_kernel  seeds and basis flows (Sec. 2.3), then the next
+//                         interval's seeds
+//      write_live_kernel, write_term_kernel  the same outputs for the tiled
+//                         list and the allocation-free interval
 //
 // Design (GB300): the hot kernel is a gather over the velocity nodes, bound
 // by memory traffic, not by arithmetic; there is no dense contraction, so the
@@ -273,6 +275,128 @@ __global__ void seed_kernel(const BlockDev *__restrict__ blocks, const int32_t *
     }
 }
 
+// K4: the end of an interval of an untiled list: basis flows (and, when
+// asked, clipped exit locations and times), termination records cleared, and
+// the next interval's seeds, in one pass over the slots. Bound by HBM. As
+// three kernels (live particles, terminated particles over all term records,
+// seeds) the pass read and wrote half as much again: 16.8M particles 319 us,
+// 270 us so; a small block's three launches become one.
+//
+// A slot's seed is perm[] of its place in the list; in a group that lost no
+// particle it is also the id the slot still holds, so perm is read, and the
+// slot's seed looked up among the terminated particles, only in the others.
+// A CTA is one region unit of 128 slots, which holds whole groups.
+struct EndArgs {
+    const BlockDev *blocks;
+    const int32_t *gblock;
+    const int32_t *perm;
+    PartList p;
+    float4 *term;
+    const float4 *clip;
+    float *seeds, *ends;
+    uint8_t *valid;
+    int32_t *exit_cycle;
+    float *exit_pos, *exit_time;
+    int32_t *err;
+    int group;
+};
+
+// Writes v of each lane to out[3 at], 12 bytes. Where the warp's particles
+// are consecutive (a full run of seeds along x), the 384 bytes go through
+// shared memory and leave as three stores of whole 128-byte lines; as three
+// 12-byte-strided stores every sector would be written three times.
+__device__ __forceinline__ void store3(float *__restrict__ out, bool on, int64_t at, const float3 v, float *stage) {
+    const int lane = threadIdx.x & 31;
+    const int64_t first = __shfl_sync(kFull, (long long)at, 0);
+    if (__all_sync(kFull, on && at == first + lane)) {
+        stage[3 * lane] = v.x;
+        stage[3 * lane + 1] = v.y;
+        stage[3 * lane + 2] = v.z;
+        __syncwarp();
+        float *o = out + 3 * first + lane;
+        o[0] = stage[lane];
+        o[32] = stage[lane + 32];
+        o[64] = stage[lane + 64];
+        __syncwarp();
+    } else if (on) {
+        out[3 * at] = v.x;
+        out[3 * at + 1] = v.y;
+        out[3 * at + 2] = v.z;
+    }
+}
+
+__global__ void __launch_bounds__(kRegionAlign) end_interval_kernel(const EndArgs a) {
+    __shared__ float stage_all[kRegionAlign / 32][96];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float *stage = stage_all[threadIdx.x >> 5];
+    const int64_t i = (int64_t)blockIdx.x * kRegionAlign + threadIdx.x;
+    // the slot's record and its group's count do not wait for the block's geometry
+    float *u = a.p.rec + part_at(i, 0);
+    const float3 xi = make_float3(__ldcs(u), __ldcs(u + 32), __ldcs(u + 64));
+    const int32_t id = __float_as_int(__ldcs(u + 96));
+    const int64_t g = i / a.group;
+    const int k = (int)(i % a.group);
+    const int cnt = a.p.gcnt[g];
+    const BlockDev &B = a.blocks[a.gblock[i / kUnit]];
+    const int64_t m = i - B.slot_base;
+    const int64_t left = B.nseeds - (m - k);
+    const int full = (int)(left < 0 ? 0 : (left > a.group ? a.group : left));   // seeds of the group
+    const float nan = __int_as_float(0x7fc00000);
+    const bool live = k < cnt && BTO_IN_BOUNDS(id >= 0 && id < B.nseeds, a.err);
+    const int64_t gid = B.base + id;
+    store3(a.ends, live, gid,
+           make_float3(fmaf(xi.x, B.h[0], B.origin[0]), fmaf(xi.y, B.h[1], B.origin[1]), fmaf(xi.z, B.h[2], B.origin[2])),
+           stage);
+    if (a.exit_pos) store3(a.exit_pos, live, gid, make_float3(nan, nan, nan), stage);
+    if (live) {
+        a.valid[gid] = 1;
+        if (a.exit_cycle) a.exit_cycle[gid] = -1;
+        if (a.exit_time) a.exit_time[gid] = nan;
+    }
+    const bool seed = m < B.nseeds;
+    int32_t p = id;
+    if (seed && (cnt != full || !live)) {
+        p = a.perm[B.base + m];
+        u[96] = __int_as_float(p);
+        const int64_t tid = B.base + p;
+        const float4 r = a.term[tid];
+        const int e = __float_as_int(r.w);
+        if (e >= 0) {
+            a.ends[3 * tid + 0] = fmaf(r.x, B.h[0], B.origin[0]);
+            a.ends[3 * tid + 1] = fmaf(r.y, B.h[1], B.origin[1]);
+            a.ends[3 * tid + 2] = fmaf(r.z, B.h[2], B.origin[2]);
+            a.valid[tid] = 0;
+            if (a.exit_cycle) a.exit_cycle[tid] = e;
+            if (a.exit_pos || a.exit_time) {
+                const float4 qs = a.clip[tid];
+                const float4 cl = clip_exit(make_float3((float)B.n[0], (float)B.n[1], (float)B.n[2]),
+                                            make_float3(r.x, r.y, r.z), make_float3(qs.x, qs.y, qs.z),
+                                            __float_as_int(qs.w), e);
+                if (a.exit_pos) {
+                    a.exit_pos[3 * tid + 0] = fmaf(cl.x, B.h[0], B.origin[0]);
+                    a.exit_pos[3 * tid + 1] = fmaf(cl.y, B.h[1], B.origin[1]);
+                    a.exit_pos[3 * tid + 2] = fmaf(cl.z, B.h[2], B.origin[2]);
+                }
+                if (a.exit_time) a.exit_time[tid] = cl.w;
+            }
+            a.term[tid] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+        }
+    }
+    const int32_t jx = p % B.S[0], jy = (p / B.S[0]) % B.S[1], jz = p / (B.S[0] * B.S[1]);
+    const float3 s = make_float3((float)(jx * B.stride), (float)(jy * B.stride), (float)(jz * B.stride));
+    store3(a.seeds, seed, B.base + p,
+           make_float3(fmaf(s.x, B.h[0], B.origin[0]), fmaf(s.y, B.h[1], B.origin[1]), fmaf(s.z, B.h[2], B.origin[2])),
+           stage);
+    if (seed) {
+        u[0] = s.x;
+        u[32] = s.y;
+        u[64] = s.z;
+    }
+    __syncthreads();   // every slot of the group has read its live count
+    if (k == 0) a.p.gcnt[g] = full;
+}
+
 // K4a: particles alive at the end of the interval.
 __global__ void write_live_kernel(const BlockDev *__restrict__ blocks,
                                   const int32_t *__restrict__ gblock, const PartList P,
@@ -469,6 +593,23 @@ cudaError_t launch_seed(const BlockDev *blocks, const int32_t *gblock, const int
                         int64_t slots, int group, PartList p, int grid, cudaStream_t s) {
     seed_kernel<<<grid, 256, 0, s>>>(blocks, gblock, perm, slots, group, p);
     return cudaGetLastError();
+}
+
+cudaError_t launch_end_interval(const BlockDev *blocks, const int32_t *gblock, const int32_t *perm, int64_t slots,
+                                int group, PartList p, float4 *term, const float4 *clip, float *seeds, float *ends,
+                                uint8_t *valid, int32_t *exit_cycle, float *exit_pos, float *exit_time, int32_t *err,
+                                cudaStream_t s) {
+    const EndArgs a{blocks, gblock, perm, p, term, clip, seeds, ends, valid, exit_cycle, exit_pos, exit_time, err, group};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(slots / kRegionAlign));
+    cfg.blockDim = dim3(kRegionAlign);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, end_interval_kernel, a);
 }
 
 cudaError_t launch_write_live(const BlockDev *blocks, const int32_t *gblock, PartList p, int64_t slots,
