@@ -235,6 +235,29 @@ bto::PartList part_list(const bto_ctx *c, int64_t first = 0) {
     return p;
 }
 
+// The launch shape of a new context (bto_set_launch and bto_autotune change
+// it), by the particles it holds; 152 SMs of 20 resident warps are meant:
+//   up to three rounds of one 32-slot unit per warp   128 threads x 1: a warp's
+//       units run one after another, and two to a warp leave the last round
+//       half empty (64^3 cells, 262,144 seeds: 183 us against 209 of 20 cycles)
+//   from 3M   256 x 4, 80 registers: four units' records are in flight at
+//       once (16.8M seeds, 10 cycles: 2.71 ms against 3.17 at 128 x 2; F4
+//       fields, 8 cycles, 2.35 against 3.07; 2.1M: 885 us against 873)
+//   from 0.75M   256 x 2, 80 registers (2.1M seeds, 20 cycles: 837 us against
+//       873; stride 2, 25 cycles, 1.49 ms against 1.52)
+//   between   128 x 2 (0.5M: 182 us against 190 at 128 x 1, 201 at 256 x 2)
+void default_shape(bto_ctx *c) {
+    const int64_t units = c->slots / bto::kUnit, resident = (int64_t)c->sm_count * 20;
+    c->nt = 128;
+    c->ppt = units <= 3 * resident ? 1 : 2;
+    c->cap = false;
+    if (c->P >= 750000) {
+        c->nt = 256;
+        c->ppt = c->P >= 3000000 ? 4 : 2;
+        c->cap = true;
+    }
+}
+
 bto_status configure_launch(bto_ctx *c) {
     const bool batched = c->nb > 1;
     c->dyn_smem = 0;
@@ -509,6 +532,7 @@ bto_status create_impl(int32_t nb, const int32_t *extents, const float *origins,
     if (e == cudaSuccess) e = cudaMemset(c->gcnt, 0, sizeof(int32_t) * units);
     if (e != cudaSuccess) { (void)cudaGetLastError(); free_ctx(c); return cuda_status(e); }
 
+    default_shape(c);
     bto_status st = configure_launch(c);
     if (st == BTO_OK) st = seed(c, 0);
     if (st == BTO_OK) st = cuda_status(cudaDeviceSynchronize());
