@@ -54,7 +54,7 @@ typedef __int128 i128;
 
 struct LPt {
     int32_t x, y, z;   // lattice coordinates relative to the query point
-    int64_t rank;
+    uint32_t rank;     // canonical lattice id; the starting points' follow the lattice's
 };
 
 // Magnitudes: window points lie within kMaxWindow of the query and the four
@@ -63,10 +63,10 @@ struct LPt {
 // below 6 * 2^36 and the lifted 4 x 4 determinant below 4 * 3 * 2^22 * 6 *
 // 2^33 < 2^63, so 64-bit integers are exact; only the ratio test's cross
 // products (two orientations) need 128 bits.
-template <class I>
-__device__ __forceinline__ int64_t det3(I a0, I a1, I a2, I b0, I b1, I b2, I c0, I c1, I c2) {
-    return a0 * ((int64_t)b1 * c2 - (int64_t)b2 * c1) - a1 * ((int64_t)b0 * c2 - (int64_t)b2 * c0) +
-           a2 * ((int64_t)b0 * c1 - (int64_t)b1 * c0);
+// The 2 x 2 minors of coordinate differences (below 2^25) are 32-bit.
+__device__ __forceinline__ int64_t det3(int32_t a0, int32_t a1, int32_t a2, int32_t b0, int32_t b1, int32_t b2,
+                                        int32_t c0, int32_t c1, int32_t c2) {
+    return (int64_t)a0 * (b1 * c2 - b2 * c1) - (int64_t)a1 * (b0 * c2 - b2 * c0) + (int64_t)a2 * (b0 * c1 - b1 * c0);
 }
 
 // orientation: determinant of the rows b - a, c - a, d - a
@@ -75,7 +75,7 @@ __device__ __forceinline__ int64_t orient(const LPt &a, const LPt &b, const LPt 
                 d.z - a.z);
 }
 
-__device__ __forceinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e);
+__device__ __noinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e);
 
 // Sign of the 5 x 5 determinant with rows (x, y, z, w, 1) of t0..t3, e
 // under the perturbed lifting: negative when e is inside the circumsphere of
@@ -112,8 +112,8 @@ __device__ __noinline__ int lifted_sign(const LPt (&t)[4], const LPt &e) {
 // five points with a non-zero cofactor decides. e's own cofactor is orient(T)
 // > 0 (outside); vertex k's is -orient(T with e in its place), e's weight at
 // that vertex, so a vertex that e has a positive weight at makes e inside.
-__device__ __forceinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e) {
-    int64_t rank = e.rank;
+__device__ __noinline__ int perturbed_sign(const LPt (&t)[4], const LPt &e) {
+    uint32_t rank = e.rank;
     int sign = 1;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -202,7 +202,7 @@ __device__ void start_tetrahedron(int64_t P, LPt (&T)[4]) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         T[k].x = far[k][0]; T[k].y = far[k][1]; T[k].z = far[k][2];
-        T[k].rank = P + k;
+        T[k].rank = (uint32_t)(P + k);
     }
     if (orient(T[0], T[1], T[2], T[3]) < 0) { const LPt s = T[0]; T[0] = T[1]; T[1] = s; }
 }
@@ -211,7 +211,7 @@ __device__ void start_tetrahedron(int64_t P, LPt (&T)[4]) {
 // point c) with squared radius r2, stays clear of every lattice plane just
 // outside the window [x0, x1] x [y0, y1] x [z0, z1] that lies inside the
 // lattice: then no lattice point outside the window is inside it.
-__device__ bool sphere_fits(const double (&ctr)[3], double r2, int3 S, int64_t cx, int64_t cy, int64_t cz,
+__device__ __noinline__ bool sphere_fits(const double (&ctr)[3], double r2, int3 S, int64_t cx, int64_t cy, int64_t cz,
                             int64_t x0, int64_t x1, int64_t y0, int64_t y1, int64_t z0, int64_t z1) {
     const double rad = sqrt(r2) * (1.0 + 1e-12) + 1e-9;
     const double lo[3] = {(double)(x0 - cx), (double)(y0 - cy), (double)(z0 - cz)};
@@ -265,38 +265,16 @@ __device__ __forceinline__ int64_t warp_max(int64_t v) {
 }
 __device__ __forceinline__ LPt shfl_xor_pt(const LPt &p, int o) {
     LPt r;
-    r.x = __shfl_xor_sync(kAll, (long long)p.x, o);
-    r.y = __shfl_xor_sync(kAll, (long long)p.y, o);
-    r.z = __shfl_xor_sync(kAll, (long long)p.z, o);
-    r.rank = __shfl_xor_sync(kAll, (long long)p.rank, o);
+    r.x = __shfl_xor_sync(kAll, p.x, o);
+    r.y = __shfl_xor_sync(kAll, p.y, o);
+    r.z = __shfl_xor_sync(kAll, p.z, o);
+    r.rank = __shfl_xor_sync(kAll, p.rank, o);
     return r;
 }
 
 __device__ __forceinline__ void positive_orientation(LPt (&t)[4]) {
     if (orient(t[0], t[1], t[2], t[3]) < 0) { const LPt s = t[0]; t[0] = t[1]; t[1] = s; }
 }
-
-// A lane's walk over a window of wx x wy x wz points in rank order: points
-// k = lane, lane + 32, ..., with offsets (x, y, z) inside the window kept
-// by additions (a window holds at most 25 x 25 or 17 x 17 x 17 points, and
-// a lattice at most 2^31, so 32-bit indices suffice).
-struct WinIter {
-    int wx, wy, k, x, y, z;
-    __device__ WinIter(int wx_, int wy_, int start) : wx(wx_), wy(wy_), k(start) {
-        x = start % wx;
-        const int q = start / wx;
-        y = q % wy;
-        z = q / wy;
-    }
-    __device__ __forceinline__ void step() {
-        k += 32;
-        x += 32;
-        while (x >= wx) {
-            x -= wx;
-            if (++y == wy) { y = 0; ++z; }
-        }
-    }
-};
 
 // Pivot rule. The first kDeepPivots pivots enter the point deepest inside
 // the circumsphere (largest r^2 - |p - c|^2 in FP32, ties to the lowest
@@ -314,14 +292,10 @@ __device__ __forceinline__ unsigned long long depth_key(float depth, int64_t ran
     const unsigned mono = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
     return ((unsigned long long)mono << 32) | (0xffffffffu - (unsigned)rank);
 }
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long w = __shfl_xor_sync(kAll, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
+// The depth a key's high word stands for.
+__device__ __forceinline__ float depth_of(unsigned hi) {
+    return __uint_as_float((hi & 0x80000000u) ? hi & 0x7fffffffu : ~hi);
 }
-
 // Lattice coordinates of the point of rank r (r < 2^31).
 __device__ __forceinline__ void rank_coords(int3 S, int64_t r, int64_t (&p)[3]) {
     const int rr = (int)r;
@@ -331,124 +305,12 @@ __device__ __forceinline__ void rank_coords(int3 S, int64_t r, int64_t (&p)[3]) 
     p[2] = q / S.y;
 }
 
-__device__ __forceinline__ unsigned gcd(unsigned a, unsigned b) {
-    while (b) { const unsigned r = a % b; a = b; b = r; }
-    return a;
-}
-
-// The walk ended with one starting point (vertex kf of T) at weight exactly
-// 0: q lies on the facet F of the other three vertices, and no window point
-// is inside the sphere through F and the far starting point. F is a facet
-// of the Delaunay triangulation of all valid points, and q's interpolant is
-// the one over F, when (a) wrapping across F to the valid window point D on
-// the other side whose sphere through F holds no other such point gives a
-// tetrahedron whose sphere holds no valid window point at all and fits in
-// the window, or (b) no valid point of the lattice lies strictly on the far
-// side of F (F is then on the hull; shown within a work limit). Either way
-// T[kf] is replaced by a valid point (D, or a vertex of F) with weight 0.
-// Spheres through F order the points beyond it (a point inside the sphere
-// through F and D comes before D), so the lanes' candidates D combine into
-// the first one in any order.
-__device__ __noinline__ bool across_facet(int3 S, const uint8_t *__restrict__ valid, int64_t cx, int64_t cy, int64_t cz,
-                             int64_t x0, int64_t x1, int64_t y0, int64_t y1, int64_t z0, int64_t z1, LPt (&T)[4],
-                             int kf) {
-    const int lane = threadIdx.x & 31;
-    const int64_t o = orient(T[0], T[1], T[2], T[3]);
-    const int wx = (int)(x1 - x0 + 1), wy = (int)(y1 - y0 + 1), W = wx * wy * (int)(z1 - z0 + 1);
-    bool far_pt = false, have = false;
-    LPt D = T[(kf + 1) & 3];
-    for (WinIter w(wx, wy, lane); w.k < W; w.step()) {
-        const int64_t x = x0 + w.x, y = y0 + w.y, z = z0 + w.z;
-        const int64_t r = lattice_rank(S, x, y, z);
-        if (!valid[r] || T[0].rank == r || T[1].rank == r || T[2].rank == r || T[3].rank == r) continue;
-        const LPt p = {(int32_t)(x - cx), (int32_t)(y - cy), (int32_t)(z - cz), r};
-        LPt u[4] = {T[0], T[1], T[2], T[3]};
-        u[kf] = p;
-        const int64_t so = orient(u[0], u[1], u[2], u[3]);
-        if (so == 0) continue;
-        if ((so > 0) == (o > 0)) { far_pt = true; continue; }
-        if (!have) { D = p; have = true; continue; }
-        LPt t4[4] = {T[0], T[1], T[2], T[3]};
-        t4[kf] = D;
-        positive_orientation(t4);
-        if (lifted_sign(t4, p) < 0) D = p;
-    }
-    far_pt = __any_sync(kAll, far_pt);
-    for (int off = 16; off > 0; off >>= 1) {
-        const LPt Do = shfl_xor_pt(D, off);
-        const bool ho = __shfl_xor_sync(kAll, (int)have, off) != 0;
-        if (!ho || Do.rank == D.rank) continue;
-        if (!have) { D = Do; have = true; continue; }
-        LPt t4[4] = {T[0], T[1], T[2], T[3]};
-        t4[kf] = D;
-        positive_orientation(t4);
-        if (lifted_sign(t4, Do) < 0) D = Do;
-    }
-    if (have) {
-        LPt t4[4] = {T[0], T[1], T[2], T[3]};
-        t4[kf] = D;
-        positive_orientation(t4);
-        bool inside = false;
-        for (WinIter w(wx, wy, lane); w.k < W && !inside; w.step()) {
-            const int64_t x = x0 + w.x, y = y0 + w.y, z = z0 + w.z;
-            const int64_t r = lattice_rank(S, x, y, z);
-            if (!valid[r] || t4[0].rank == r || t4[1].rank == r || t4[2].rank == r || t4[3].rank == r) continue;
-            const LPt p = {(int32_t)(x - cx), (int32_t)(y - cy), (int32_t)(z - cz), r};
-            inside = lifted_sign(t4, p) < 0;
-        }
-        inside = __any_sync(kAll, inside);
-        double ctr[3], r2;
-        circumsphere(t4, ctr, r2);
-        if (!inside && sphere_fits(ctr, r2, S, cx, cy, cz, x0, x1, y0, y1, z0, z1)) {
-            T[kf] = D;
-            return true;
-        }
-    }
-    // (b): no valid point of the lattice strictly on the far side of F. The
-    // orientation with p in place of the starting point is affine in p,
-    // n.p + d, so each lattice row holds its far-side points in one interval
-    // and only those are visited (within kHullScanWork rows and points).
-    if (!far_pt) {
-        LPt u[4] = {T[0], T[1], T[2], T[3]};
-        const LPt o0 = {0, 0, 0, -1}, ex = {1, 0, 0, -1}, ey = {0, 1, 0, -1}, ez = {0, 0, 1, -1};
-        u[kf] = o0;
-        const int64_t d = orient(u[0], u[1], u[2], u[3]);
-        u[kf] = ex;
-        const int64_t nx = orient(u[0], u[1], u[2], u[3]) - d;
-        u[kf] = ey;
-        const int64_t ny = orient(u[0], u[1], u[2], u[3]) - d;
-        u[kf] = ez;
-        const int64_t nz = orient(u[0], u[1], u[2], u[3]) - d;
-        const int64_t sg = o > 0 ? 1 : -1;
-        const int64_t rows = (int64_t)S.y * S.z, budget = kHullScanWork / 32;
-        int64_t work = 0;
-        bool stop = false;                          // a far-side valid point, or out of budget
-        // Each lane keeps the rows lane, lane + 32, ...; it takes them in the
-        // order of multiples of a number coprime to their count, and the warp
-        // ends as soon as one lane has stopped: a valid point on the far side
-        // is mostly met within a few rows spread over the lattice.
-        const unsigned per = (unsigned)((rows + 31) / 32);
-        unsigned hop = per * 5 / 8 + 1;
-        while (gcd(hop, per) != 1) ++hop;
-        unsigned at = 0;
-        for (unsigned k = 0; k < per && !__any_sync(kAll, stop); ++k, at = (at + hop) % per) {
-            const int64_t row = lane + 32ll * at;
-            if (row >= rows) continue;
-            const int64_t y = (int)row % S.y, z = (int)row / S.y;
-            if (++work > budget) { stop = true; continue; }
-            int64_t t0, t1;
-            if (!positive_range(sg * nx, sg * (ny * (y - cy) + nz * (z - cz) + d), -cx, (int64_t)S.x - 1 - cx, t0, t1))
-                continue;
-            for (int64_t t = t0; t <= t1; ++t) {
-                if (++work > budget || valid[lattice_rank(S, t + cx, y, z)]) { stop = true; break; }
-            }
-        }
-        if (__any_sync(kAll, stop)) return false;
-        T[kf] = T[(kf + 1) & 3];
-        return true;
-    }
-    return false;
-}
+// x^2 + y^2 (+ z^2) of the filter and the depths, its roundings fixed: where q
+// lies on a face of several Delaunay simplices, which of them a walk ends in,
+// and with it whether the sphere fits a small window, hangs on the pivots
+// taken, and those on FP32 depths that differ in the last bit.
+__device__ __forceinline__ float sum2(float x, float y) { return __fmaf_rn(x, x, __fmul_rn(y, y)); }
+__device__ __forceinline__ float sum3(float x, float y, float z) { return __fmaf_rn(z, z, sum2(x, y)); }
 
 // The lifted plane through T and its circumsphere. For a point p of the
 // window (coordinates relative to q)
@@ -470,24 +332,22 @@ struct Sphere {
     float c[3], r2;
 };
 
-// The four determinants are shared out, one to a lane, and exchanged.
+// The four determinants are shared out, one to a lane, and exchanged; each is
+// expanded along the column that the squared lengths replace (the first, for
+// d), whose cofactors are 32-bit minors.
 __device__ __forceinline__ Sphere sphere_of(const LPt (&T)[4]) {
     const int j = threadIdx.x & 3;
-    int32_t A[3][3], b[3];
+    int32_t v[3], p[3], q[3];   // the column expanded, and the next two in cyclic order
     const LPt &a = T[0];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-        const LPt &p = T[m + 1];
-        A[m][0] = p.x - a.x;
-        A[m][1] = p.y - a.y;
-        A[m][2] = p.z - a.z;
-        b[m] = A[m][0] * A[m][0] + A[m][1] * A[m][1] + A[m][2] * A[m][2];
+        const int32_t x = T[m + 1].x - a.x, y = T[m + 1].y - a.y, z = T[m + 1].z - a.z;
+        v[m] = j == 0 ? x : x * x + y * y + z * z;
+        p[m] = j == 2 ? z : (j == 3 ? x : y);
+        q[m] = j == 2 ? x : (j == 3 ? y : z);
     }
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-#pragma unroll
-        for (int s = 0; s < 3; ++s) A[m][s] = j == s + 1 ? b[m] : A[m][s];
-    const int64_t det = det3(A[0][0], A[0][1], A[0][2], A[1][0], A[1][1], A[1][2], A[2][0], A[2][1], A[2][2]);
+    const int64_t det = (int64_t)v[0] * (p[1] * q[2] - q[1] * p[2]) + (int64_t)v[1] * (p[2] * q[0] - q[2] * p[0]) +
+                        (int64_t)v[2] * (p[0] * q[1] - q[0] * p[1]);
     Sphere S;
     S.d = __shfl_sync(kAll, (long long)det, 0);
     int64_t n[3];
@@ -506,19 +366,25 @@ __device__ __forceinline__ Sphere sphere_of(const LPt (&T)[4]) {
         u[s] = 0.5f * ((float)n[s] / fd);
         S.c[s] = u[s] + (float)ac[s];
     }
-    S.r2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    S.r2 = sum3(u[0], u[1], u[2]);
     return S;
+}
+
+// F(p) (see Sphere).
+__device__ __forceinline__ int64_t sphere_value(const Sphere &S, const LPt &p) {
+    return (int64_t)((uint64_t)S.d * (uint64_t)(int64_t)(p.x * p.x + p.y * p.y + p.z * p.z) -
+                     S.m[0] * (uint64_t)(int64_t)p.x - S.m[1] * (uint64_t)(int64_t)p.y -
+                     S.m[2] * (uint64_t)(int64_t)p.z + S.k);
 }
 
 // Whether the window point p (of rank r) is inside the circumsphere of T
 // under the perturbed lifting; false for T's own vertices.
 __device__ __forceinline__ bool inside_sphere(const Sphere &S, const LPt (&T)[4], const LPt &p) {
-    const int64_t F = (int64_t)((uint64_t)S.d * (uint64_t)(int64_t)(p.x * p.x + p.y * p.y + p.z * p.z) -
-                                S.m[0] * (uint64_t)(int64_t)p.x - S.m[1] * (uint64_t)(int64_t)p.y -
-                                S.m[2] * (uint64_t)(int64_t)p.z + S.k);
+    const int64_t F = sphere_value(S, p);
     if (F != 0) return F < 0;
     if (T[0].rank == p.rank || T[1].rank == p.rank || T[2].rank == p.rank || T[3].rank == p.rank) return false;
-    return perturbed_sign(T, p) < 0;
+    const LPt t4[4] = {T[0], T[1], T[2], T[3]};   // the copy keeps T itself in registers
+    return perturbed_sign(t4, p) < 0;
 }
 
 // The valid points around a tile of kTileX x kTileY x kTileZ entries, one
@@ -526,9 +392,168 @@ __device__ __forceinline__ bool inside_sphere(const Sphere &S, const LPt (&T)[4]
 // (x0 + k, y0 + ry, z0 + rz), (x0, y0, z0) the tile's first entry less
 // kMaxWindow per axis. Every entry of the tile reads its whole window from
 // these words, 17 bits a row, instead of a byte of memory per point.
-constexpr int kTileX = 16, kTileY = 4, kTileZ = 4;
+constexpr int kTileX = 8, kTileY = 2, kTileZ = 2;
 constexpr int kRowsY = kTileY + 2 * kMaxWindow, kRowsZ = kTileZ + 2 * kMaxWindow;
-static_assert(kTileX + 2 * kMaxWindow == 32, "a row of the tile's surroundings is one word");
+static_assert(kTileX + 2 * kMaxWindow <= 32, "a row of the tile's surroundings is one word");
+
+// The bits of a window row at or below the x of the centre c0 (x = bit -
+// kMaxWindow); the row's points fall off in depth outward from there on both
+// sides. Where FP32 rounds c0 across a point, that point is the nearest on
+// either reading.
+__device__ __forceinline__ uint32_t bits_below(float c0) {
+    const int split = (int)fminf(fmaxf(floorf(c0), -(float)(kMaxWindow + 1)), (float)kMaxWindow) + kMaxWindow;
+    return split < 0 ? 0u : (2u << split) - 1u;
+}
+
+__device__ __forceinline__ unsigned gcd(unsigned a, unsigned b) {
+    while (b) { const unsigned r = a % b; a = b; b = r; }
+    return a;
+}
+
+// The walk ended with one starting point (vertex kf of T) at weight exactly
+// 0: q lies on the facet F of the other three vertices, and no window point
+// is inside the sphere through F and the far starting point. F is a facet
+// of the Delaunay triangulation of all valid points, and q's interpolant is
+// the one over F, when (a) wrapping across F to the valid window point D on
+// the other side whose sphere through F holds no other such point gives a
+// tetrahedron whose sphere holds no valid window point at all and fits in
+// the window, or (b) no valid point of the lattice lies strictly on the far
+// side of F (F is then on the hull; shown within a work limit). Either way
+// T[kf] is replaced by a valid point (D, or a vertex of F) with weight 0.
+// Spheres through F order the points beyond it (a point inside the sphere
+// through F and D comes before D), so the lanes' candidates D combine into
+// the first one in any order.
+__device__ __noinline__ bool across_facet(int3 S, const uint8_t *__restrict__ valid, const uint32_t *win, int lx, int cx,
+                                          int cy, int cz, int R, LPt (&T)[4], int kf) {
+    const int lane = threadIdx.x & 31;
+    const int side = 2 * R + 1, rows_w = side * side;
+    const uint32_t wmask = ((1u << side) - 1u) << (kMaxWindow - R);
+    const int64_t x0 = max(cx - R, 0), x1 = min(cx + R, S.x - 1), y0 = max(cy - R, 0), y1 = min(cy + R, S.y - 1),
+                  z0 = max(cz - R, 0), z1 = min(cz + R, S.z - 1);
+    // h(p) = orient(T) with p in the starting point's place = nx x + ny y + nz z + d: positive on its side of F
+    LPt u[4];
+    const LPt o0 = {0, 0, 0, 0}, ex = {1, 0, 0, 0}, ey = {0, 1, 0, 0}, ez = {0, 0, 1, 0};
+    auto with = [&](const LPt &p) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) u[k] = k == kf ? p : T[k];
+        return orient(u[0], u[1], u[2], u[3]);
+    };
+    const int64_t d = with(o0), nx = with(ex) - d, ny = with(ey) - d, nz = with(ez) - d;
+    // F's spheres order the points beyond it by F(p) / |h(p)|, F(p) the value
+    // of T's own sphere: the sphere through F and p holds the points whose
+    // quotient is smaller. FP32 quotients (three roundings) decide unless
+    // they are within 1e-5 of each other, the exact predicate otherwise.
+    const Sphere sp = sphere_of(T);
+    bool far_pt = false, have = false;
+    LPt D = o0;
+    float Dq = 0.f;
+    auto closer = [&](const LPt &p) {   // p inside the sphere through F and D
+        LPt t4[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t4[k] = k == kf ? D : T[k];
+        positive_orientation(t4);
+        return lifted_sign(t4, p) < 0;
+    };
+#pragma unroll 1
+    for (int row = lane; row < rows_w; row += 32) {
+        const int rz = row / side, dy = row - rz * side - R, dz = rz - R;
+        uint32_t m = (win[dy + kRowsY * dz] >> lx) & wmask;
+        const int r0 = cx - kMaxWindow + S.x * (cy + dy + S.y * (cz + dz));
+#pragma unroll 1
+        while (m) {
+            const int bit = __ffs(m) - 1;
+            m &= m - 1;
+            const LPt p = {bit - kMaxWindow, dy, dz, (uint32_t)(r0 + bit)};
+            const int64_t h = nx * p.x + ny * dy + nz * dz + d;
+            if (h == 0) continue;   // F's own vertices among them
+            if (h > 0) { far_pt = true; continue; }
+            const float q = (float)sphere_value(sp, p) / (float)(-h);
+            if (!have || q < Dq * 0.99999f || (q <= Dq * 1.00001f && closer(p))) { D = p; Dq = q; have = true; }
+        }
+    }
+    far_pt = __any_sync(kAll, far_pt);
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) {
+        const LPt Do = shfl_xor_pt(D, off);
+        const float qo = __shfl_xor_sync(kAll, Dq, off);
+        const bool ho = __shfl_xor_sync(kAll, (int)have, off) != 0;
+        if (!ho || (have && Do.rank == D.rank)) continue;
+        if (!have || closer(Do)) { D = Do; Dq = qo; have = true; }
+    }
+    if (have) {
+        LPt t4[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t4[k] = k == kf ? D : T[k];
+        positive_orientation(t4);
+        const Sphere s4 = sphere_of(t4);
+        const uint32_t lowbits = bits_below(s4.c[0]);
+        bool inside = false;
+#pragma unroll 1
+        for (int row = lane; row < rows_w && !inside; row += 32) {
+            const int rz = row / side, dy = row - rz * side - R, dz = rz - R;
+            const uint32_t m = (win[dy + kRowsY * dz] >> lx) & wmask;
+            const int r0 = cx - kMaxWindow + S.x * (cy + dy + S.y * (cz + dz));
+            // the nearest point on each side; the others of the row are
+            // farther out, and strictly outside unless it is inside
+            const uint32_t lo = m & lowbits, hi = m & ~lowbits;
+#pragma unroll 1
+            for (int dir = 0; dir < 2 && !inside; ++dir) {
+                if (!(dir ? hi : lo)) continue;
+                const int bit = dir ? __ffs(hi) - 1 : 31 - __clz(lo);
+                const LPt p = {bit - kMaxWindow, dy, dz, (uint32_t)(r0 + bit)};
+                inside = inside_sphere(s4, t4, p);
+            }
+        }
+        inside = __any_sync(kAll, inside);
+        if (!inside) {
+            double ctr[3], r2;
+            circumsphere(t4, ctr, r2);
+            if (sphere_fits(ctr, r2, S, cx, cy, cz, x0, x1, y0, y1, z0, z1)) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (k == kf) T[k] = D;
+                return true;
+            }
+        }
+    }
+    // (b): no valid point of the lattice strictly on the far side of F. The
+    // orientation with p in place of the starting point is affine in p,
+    // n.p + d, so each lattice row holds its far-side points in one interval
+    // and only those are visited (within kHullScanWork rows and points).
+    if (!far_pt) {
+        const int64_t rows = (int64_t)S.y * S.z, budget = kHullScanWork / 32;
+        int64_t work = 0;
+        bool stop = false;                          // a far-side valid point, or out of budget
+        // Each lane keeps the rows lane, lane + 32, ...; it takes them in the
+        // order of multiples of a number coprime to their count, and the warp
+        // ends as soon as one lane has stopped: a valid point on the far side
+        // is mostly met within a few rows spread over the lattice.
+        const unsigned per = (unsigned)((rows + 31) / 32);
+        unsigned hop = per * 5 / 8 + 1;
+        while (gcd(hop, per) != 1) ++hop;
+        unsigned at = 0;
+        for (unsigned k = 0; k < per && !__any_sync(kAll, stop); ++k, at = (at + hop) % per) {
+            const int64_t row = lane + 32ll * at;
+            if (row >= rows) continue;
+            const int64_t y = (int)row % S.y, z = (int)row / S.y;
+            if (++work > budget) { stop = true; continue; }
+            int64_t t0, t1;
+            if (!positive_range(nx, ny * (y - cy) + nz * (z - cz) + d, -(int64_t)cx, (int64_t)S.x - 1 - cx, t0, t1))
+                continue;
+#pragma unroll 1
+            for (int64_t t = t0; t <= t1; ++t) {
+                if (++work > budget || valid[lattice_rank(S, t + cx, y, z)]) { stop = true; break; }
+            }
+        }
+        if (__any_sync(kAll, stop)) return false;
+        const LPt other = kf == 3 ? T[0] : (kf == 0 ? T[1] : (kf == 1 ? T[2] : T[3]));
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k == kf) T[k] = other;
+        return true;
+    }
+    return false;
+}
 
 // One walk in the window of radius R around c, from the tetrahedron T it is
 // given (a feasible basis: q inside it), so a larger window resumes where a
@@ -551,24 +576,54 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
     const uint32_t wmask = ((1u << side) - 1u) << (kMaxWindow - R);
     const uint32_t ends = (1u << (kMaxWindow - R)) | (1u << (kMaxWindow + R));
     const unsigned inv_side = 65536u / (unsigned)side + 1u;   // row / side for rows < 2^16 / side
+#pragma unroll 1
     for (int it = 0; it < kMaxPivots; ++it) {
         // entering point: among the valid window points inside the
-        // circumsphere of T, the deepest (later the lowest-ranked) one. A
-        // point clearly outside by its FP32 distance to the centre is
-        // skipped: near the sphere the squared distance's rounding error
-        // stays below 2e-6 r^2, so with the margin 1e-4 r^2 + 1e-2 only
-        // points strictly outside are skipped; every other candidate gets
-        // the exact predicate, so the choice is the exact one.
+        // circumsphere of T, the deepest (later the lowest-ranked) one. Near
+        // the sphere the FP32 squared distance's rounding error stays below
+        // 2e-6 r^2; a point farther than 8e-6 r^2 + 1e-3 from it is inside
+        // or outside for certain. Most pivots enter a point that is inside
+        // for certain, found from the nearest points of each row alone;
+        // otherwise the candidates in the margin get the exact predicate.
         const Sphere sp = sphere_of(T);
         const float fc0 = sp.c[0], fc1 = sp.c[1], fc2 = sp.c[2];
-        const float fr2 = sp.r2 * (1.0f + 1e-4f) + 1e-2f;
+        const float margin = sp.r2 * 8e-6f + 1e-3f, fr2 = sp.r2 + margin;
         const bool deep = it < kDeepPivots, shell = settled && it == 0;
-        // bits up to `split` lie at or below the centre's x
-        const int split = (int)fminf(fmaxf(floorf(fc0), -(float)(kMaxWindow + 1)), (float)kMaxWindow) + kMaxWindow;
-        const uint32_t lowbits = split < 0 ? 0u : (2u << split) - 1u;
+        const uint32_t lowbits = bits_below(fc0);
         int64_t best = kNone;
         unsigned bhi = 0, blo = 0;   // the lane's best depth key (depth_key), 0: none
-        for (int row = lane; row < rows; row += 32) {
+        if (deep) {
+#pragma unroll 1
+            for (int row = lane; row < rows; row += 32) {
+                const int rz = (int)(((unsigned)row * inv_side) >> 16), dy = row - rz * side - R, dz = rz - R;
+                uint32_t m = (win[dy + kRowsY * dz] >> lx) & wmask;
+                if (shell && dy > -R && dy < R && dz > -R && dz < R) m &= ends;
+                const uint32_t lo = m & lowbits, hi = m & ~lowbits;
+                const float fy = (float)dy - fc1, fz = (float)dz - fc2;
+                const int r0 = cx - kMaxWindow + S.x * (cy + dy + S.y * (cz + dz));
+#pragma unroll 1
+                for (int dir = 0; dir < 2; ++dir) {
+                    uint32_t w = dir ? hi : lo;
+#pragma unroll 1
+                    while (w) {
+                        const int bit = dir ? __ffs(w) - 1 : 31 - __clz(w);
+                        w &= ~(1u << bit);
+                        const float fx = (float)(bit - kMaxWindow) - fc0;
+                        const unsigned long long key = depth_key(sp.r2 - (sum3(fx, fy, fz)), r0 + bit);
+                        const unsigned khi = (unsigned)(key >> 32), klo = (unsigned)key;
+                        if (khi < bhi || (khi == bhi && klo <= blo)) break;
+                        bhi = khi;
+                        blo = klo;
+                        if (dir) break;   // FP32 depth can be level along a row: the lowest rank is the one to keep
+                    }
+                }
+            }
+        }
+        const unsigned sure = __reduce_max_sync(kAll, bhi);
+        const bool clear = deep && sure != 0 && depth_of(sure) > margin;
+        if (!clear) { bhi = 0; blo = 0; }
+#pragma unroll 1
+        for (int row = clear ? rows : lane; row < rows; row += 32) {
             const int rz = (int)(((unsigned)row * inv_side) >> 16), dy = row - rz * side - R, dz = rz - R;
             uint32_t m = (win[dy + kRowsY * dz] >> lx) & wmask;
             if (shell && dy > -R && dy < R && dz > -R && dz < R) m &= ends;
@@ -576,22 +631,23 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
             const float fy = (float)dy - fc1, fz = (float)dz - fc2;
             const int r0 = cx - kMaxWindow + S.x * (cy + dy + S.y * (cz + dz));   // the row's ranks are r0 + bit, below 2^31
             if (deep) {
-#pragma unroll
+#pragma unroll 1
                 for (int dir = 0; dir < 2; ++dir) {
                     uint32_t w = dir ? m & ~lowbits : m & lowbits;
+#pragma unroll 1
                     while (w) {
                         const int bit = dir ? __ffs(w) - 1 : 31 - __clz(w);
                         w &= ~(1u << bit);
                         const int dx = bit - kMaxWindow;
                         const float fx = (float)dx - fc0;
-                        const float d2 = fx * fx + fy * fy + fz * fz;
+                        const float d2 = sum3(fx, fy, fz);
                         if (d2 > fr2) break;
                         const int r = r0 + bit;
                         const unsigned long long key = depth_key(sp.r2 - d2, r);
                         const unsigned khi = (unsigned)(key >> 32), klo = (unsigned)key;
                         if (khi < bhi) break;
                         if (khi == bhi && klo <= blo) continue;
-                        const LPt p = {dx, dy, dz, r};
+                        const LPt p = {dx, dy, dz, (uint32_t)r};
                         if (inside_sphere(sp, T, p)) {
                             bhi = khi;
                             blo = klo;
@@ -604,8 +660,8 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
                     m &= m - 1;
                     const int dx = bit - kMaxWindow;
                     const float fx = (float)dx - fc0;
-                    if (fx * fx + fy * fy + fz * fz > fr2) continue;
-                    const LPt p = {dx, dy, dz, r0 + bit};
+                    if (sum3(fx, fy, fz) > fr2) continue;
+                    const LPt p = {dx, dy, dz, (uint32_t)(r0 + bit)};
                     if (inside_sphere(sp, T, p)) best = r0 + bit;
                 }
                 if (best != kNone) break;
@@ -621,16 +677,16 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
         // orientations with vertex k replaced, one vertex to a lane (lanes
         // 4 apart hold the same): by q (oq) and, when a point enters, by
         // that point (oe)
-        const LPt q0 = {0, 0, 0, -1};
+        const LPt q0 = {0, 0, 0, 0};
         const int mine = lane & 3;
         LPt u[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) u[k] = mine == k ? q0 : T[k];
         const int64_t oq = orient(u[0], u[1], u[2], u[3]);
-        const int64_t rank_mine = mine == 0 ? T[0].rank : (mine == 1 ? T[1].rank : (mine == 2 ? T[2].rank : T[3].rank));
+        const uint32_t rank_mine = mine == 0 ? T[0].rank : (mine == 1 ? T[1].rank : (mine == 2 ? T[2].rank : T[3].rank));
         if (best == kNone) {
             settled = true;
-            const unsigned far = __ballot_sync(kAll, rank_mine >= P) & 15u;
+            const unsigned far = __ballot_sync(kAll, rank_mine >= (uint32_t)P) & 15u;
             const unsigned zero = __ballot_sync(kAll, oq == 0) & 15u;
             if (far == 0) {
                 // the circumsphere must fit in the window: then no lattice
@@ -656,7 +712,7 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
             if (far == 0) return 1;
             // a starting point with weight 0: q is on a facet
             LPt t4[4] = {T[0], T[1], T[2], T[3]};
-            if (!across_facet(S, valid, cx, cy, cz, x0, x1, y0, y1, z0, z1, t4, __ffs(far) - 1)) return 0;
+            if (!across_facet(S, valid, win, lx, cx, cy, cz, R, t4, __ffs(far) - 1)) return 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) T[k] = t4[k];
             return 1;
@@ -664,7 +720,7 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
         settled = false;
         const unsigned b32 = (unsigned)best;
         const int ez = (int)(b32 / (unsigned)(S.x * S.y)), ey = (int)(b32 / (unsigned)S.x) - ez * S.y;
-        const LPt e = {(int32_t)(b32 % (unsigned)S.x) - cx, ey - cy, ez - cz, best};
+        const LPt e = {(int32_t)(b32 % (unsigned)S.x) - cx, ey - cy, ez - cz, b32};
 #pragma unroll
         for (int k = 0; k < 4; ++k) u[k] = mine == k ? e : T[k];
         const int64_t oe = orient(u[0], u[1], u[2], u[3]);
@@ -680,7 +736,8 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
         const unsigned near = __ballot_sync(kAll, ratio <= least * 1.00001f) & 15u;
         int leave = __ffs(near) - 1;
         if (near & (near - 1)) {
-            int64_t bq = 0, be = 0, brank = 0;
+            int64_t bq = 0, be = 0;
+            uint32_t brank = 0;
             leave = -1;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -711,7 +768,7 @@ __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, c
 
 struct LPt2 {
     int32_t u, v;      // free coordinates relative to the query point
-    int64_t rank;
+    uint32_t rank;
 };
 
 // Counter-clockwise orientation of (a, b, c): positive when counter-clockwise.
@@ -735,7 +792,10 @@ __device__ __forceinline__ int lifted_sign2(const LPt2 (&t)[3], const LPt2 &e) {
         r[i][1] = t[i].v - e.v;
         r[i][2] = r[i][0] * r[i][0] + r[i][1] * r[i][1];
     }
-    const int64_t d0 = det3(r[0][0], r[0][1], r[0][2], r[1][0], r[1][1], r[1][2], r[2][0], r[2][1], r[2][2]);
+    // expanded along the squared lengths
+    const int64_t d0 = (int64_t)r[0][2] * (r[1][0] * r[2][1] - r[1][1] * r[2][0]) -
+                       (int64_t)r[1][2] * (r[0][0] * r[2][1] - r[0][1] * r[2][0]) +
+                       (int64_t)r[2][2] * (r[0][0] * r[1][1] - r[0][1] * r[1][0]);
     if (d0 != 0) return d0 > 0 ? 1 : -1;
     return perturbed_sign2(t, e);
 }
@@ -743,7 +803,7 @@ __device__ __forceinline__ int lifted_sign2(const LPt2 (&t)[3], const LPt2 &e) {
 // The sign when the unperturbed determinant is zero, as perturbed_sign: e's
 // own cofactor says outside, vertex k's has the sign of e's weight there.
 __device__ __forceinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e) {
-    int64_t rank = e.rank;
+    uint32_t rank = e.rank;
     int sign = -1;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -781,7 +841,7 @@ __device__ __forceinline__ void circumcircle_f(const LPt2 (&T)[3], float (&c)[2]
     const float ux = (float)(cy * b2 - by * c2) / d, uy = (float)(bx * c2 - cx * b2) / d;
     c[0] = ux + (float)T[0].u;
     c[1] = uy + (float)T[0].v;
-    r2 = ux * ux + uy * uy;
+    r2 = sum2(ux, uy);
 }
 
 // Sets T to three far starting points around q (counter-clockwise).
@@ -790,7 +850,7 @@ __device__ void start_triangle(int64_t P, LPt2 (&T)[3]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         T[k].u = far[k][0]; T[k].v = far[k][1];
-        T[k].rank = P + k;
+        T[k].rank = (uint32_t)(P + k);
     }
     if (orient2(T[0], T[1], T[2]) < 0) { const LPt2 s = T[0]; T[0] = T[1]; T[1] = s; }
 }
@@ -812,94 +872,137 @@ __device__ bool circle_fits(const double (&ctr)[2], double r2, int3 S, const int
     return true;
 }
 
+// A face's entry and its window, one row (fixed v) to a lane: bit k of
+// lane l's word is the face's point (k - kMaxWindow2, l - kMaxWindow2) in
+// the free axes a < b, relative to the entry.
+struct Face {
+    int a, b;          // free axes
+    int ca, cb;        // the entry's coordinates along them
+    int ea, eb;        // lattice extents along them
+    int sa, sb;        // rank steps along them
+    int rq;            // the entry's rank
+    uint32_t row;      // the lane's word
+};
+static_assert(2 * kMaxWindow2 + 1 <= 32, "a face's window is one word per lane");
+
+__device__ __forceinline__ Face face_of(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], int a, int b) {
+    Face f;
+    f.a = a;
+    f.b = b;
+    // a is 0 or 1, b is 1 or 2
+    f.ca = (int)(a == 0 ? c[0] : c[1]);
+    f.cb = (int)(b == 1 ? c[1] : c[2]);
+    f.ea = a == 0 ? S.x : S.y;
+    f.eb = b == 1 ? S.y : S.z;
+    f.sa = a == 0 ? 1 : S.x;
+    f.sb = b == 1 ? S.x : S.x * S.y;
+    f.rq = (int)lattice_rank(S, c[0], c[1], c[2]);
+    const int lane = threadIdx.x & 31, du = lane - kMaxWindow2;
+    const bool in_u = lane <= 2 * kMaxWindow2 && f.ca + du >= 0 && f.ca + du < f.ea;
+    f.row = 0;
+#pragma unroll 5
+    for (int k = 0; k <= 2 * kMaxWindow2; ++k) {
+        const int dv = k - kMaxWindow2;
+        const bool in = in_u && f.cb + dv >= 0 && f.cb + dv < f.eb;
+        const unsigned w = __ballot_sync(kAll, in && valid[f.rq + du * f.sa + dv * f.sb] != 0);
+        if (lane == k) f.row = w;
+    }
+    return f;
+}
+
+// The lane's row cut to the window of radius R.
+__device__ __forceinline__ uint32_t face_row(const Face &f, int R) {
+    const int dv = (int)(threadIdx.x & 31) - kMaxWindow2;
+    return abs(dv) <= R ? f.row & (((2u << (2 * R)) - 1u) << (kMaxWindow2 - R)) : 0u;
+}
+
 // across_facet on a face: q lies on the edge F opposite the starting point
 // T[kf] (weight exactly 0). Wrap across F to the valid window point D whose
 // circle through F holds no other point on that side; accept when that
 // triangle's circle holds no valid window point and fits in the window, or
 // when no valid point of the face lies strictly on the far side of F (F is
 // then on the hull of the face's points).
-__device__ __noinline__ bool across_edge(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], int a, int b,
-                            int64_t u0, int64_t u1, int64_t v0, int64_t v1, LPt2 (&T)[3], int kf) {
-    const int lane = threadIdx.x & 31;
-    const int64_t ext[3] = {S.x, S.y, S.z};
-    const LPt2 A = T[(kf + 1) % 3], B = T[(kf + 2) % 3];
-    const int64_t sf = orient2(A, B, T[kf]);
-    const int wu = (int)(u1 - u0 + 1), W = wu * (int)(v1 - v0 + 1);
+__device__ __noinline__ bool across_edge(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], const Face &f,
+                                         int R, LPt2 (&T)[3], int kf) {
+    const int lane = threadIdx.x & 31, dv = lane - kMaxWindow2;
+    const LPt2 A = kf == 0 ? T[1] : (kf == 1 ? T[2] : T[0]), B = kf == 0 ? T[2] : (kf == 1 ? T[0] : T[1]);
+    const LPt2 far = kf == 0 ? T[0] : (kf == 1 ? T[1] : T[2]);
+    const int64_t sf = orient2(A, B, far);
+    const uint32_t row = face_row(f, R);
+    const int r0 = f.rq + dv * f.sb - kMaxWindow2 * f.sa;   // the rank of bit k is r0 + k sa
     bool far_pt = false, have = false;
     LPt2 D = A;
-    for (WinIter w(wu, 1 << 30, lane); w.k < W; w.step()) {
-        int64_t pc[3] = {c[0], c[1], c[2]};
-        pc[a] = u0 + w.x;
-        pc[b] = v0 + w.y;
-        const int64_t r = lattice_rank(S, pc[0], pc[1], pc[2]);
-        if (!valid[r] || r == A.rank || r == B.rank) continue;
-        const LPt2 p = {(int32_t)(pc[a] - c[a]), (int32_t)(pc[b] - c[b]), r};
+    auto closer = [&](const LPt2 &p) {   // p inside the circle through F and D
+        const bool ccw = orient2(A, B, D) >= 0;
+        const LPt2 t3[3] = {ccw ? A : B, ccw ? B : A, D};
+        return lifted_sign2(t3, p) > 0;
+    };
+    for (uint32_t m = row; m; m &= m - 1) {
+        const int k = __ffs(m) - 1;
+        const LPt2 p = {k - kMaxWindow2, dv, (uint32_t)(r0 + k * f.sa)};
+        if (p.rank == A.rank || p.rank == B.rank) continue;
         const int64_t so = orient2(A, B, p);
         if (so == 0) continue;
         if ((so > 0) == (sf > 0)) { far_pt = true; continue; }
-        if (!have) { D = p; have = true; continue; }
-        LPt2 t3[3] = {A, B, D};
-        if (orient2(t3[0], t3[1], t3[2]) < 0) { const LPt2 sw = t3[0]; t3[0] = t3[1]; t3[1] = sw; }
-        if (lifted_sign2(t3, p) > 0) D = p;
+        if (!have || closer(p)) { D = p; have = true; }
     }
     far_pt = __any_sync(kAll, far_pt);
     for (int off = 16; off > 0; off >>= 1) {
         LPt2 Do;
-        Do.u = __shfl_xor_sync(kAll, (long long)D.u, off);
-        Do.v = __shfl_xor_sync(kAll, (long long)D.v, off);
-        Do.rank = __shfl_xor_sync(kAll, (long long)D.rank, off);
+        Do.u = __shfl_xor_sync(kAll, D.u, off);
+        Do.v = __shfl_xor_sync(kAll, D.v, off);
+        Do.rank = __shfl_xor_sync(kAll, D.rank, off);
         const bool ho = __shfl_xor_sync(kAll, (int)have, off) != 0;
-        if (!ho || Do.rank == D.rank) continue;
-        if (!have) { D = Do; have = true; continue; }
-        LPt2 t3[3] = {A, B, D};
-        if (orient2(t3[0], t3[1], t3[2]) < 0) { const LPt2 sw = t3[0]; t3[0] = t3[1]; t3[1] = sw; }
-        if (lifted_sign2(t3, Do) > 0) D = Do;
+        if (!ho || (have && Do.rank == D.rank)) continue;
+        if (!have || closer(Do)) { D = Do; have = true; }
     }
     if (have) {
-        LPt2 t3[3] = {A, B, D};
-        if (orient2(t3[0], t3[1], t3[2]) < 0) { const LPt2 sw = t3[0]; t3[0] = t3[1]; t3[1] = sw; }
         bool inside = false;
-        for (WinIter w(wu, 1 << 30, lane); w.k < W && !inside; w.step()) {
-            int64_t pc[3] = {c[0], c[1], c[2]};
-            pc[a] = u0 + w.x;
-            pc[b] = v0 + w.y;
-            const int64_t r = lattice_rank(S, pc[0], pc[1], pc[2]);
-            if (!valid[r] || r == A.rank || r == B.rank || r == D.rank) continue;
-            const LPt2 p = {(int32_t)(pc[a] - c[a]), (int32_t)(pc[b] - c[b]), r};
-            inside = lifted_sign2(t3, p) > 0;
+        for (uint32_t m = row; m && !inside; m &= m - 1) {
+            const int k = __ffs(m) - 1;
+            const LPt2 p = {k - kMaxWindow2, dv, (uint32_t)(r0 + k * f.sa)};
+            if (p.rank == A.rank || p.rank == B.rank || p.rank == D.rank) continue;
+            inside = closer(p);
         }
         inside = __any_sync(kAll, inside);
-        double ctr[2], r2;
-        circumcircle(t3, ctr, r2);
-        if (!inside && circle_fits(ctr, r2, S, c, a, b, u0, u1, v0, v1)) {
-            T[kf] = D;
-            return true;
+        if (!inside) {
+            const bool ccw = orient2(A, B, D) >= 0;
+            const LPt2 t3[3] = {ccw ? A : B, ccw ? B : A, D};
+            double ctr[2], r2;
+            circumcircle(t3, ctr, r2);
+            if (circle_fits(ctr, r2, S, c, f.a, f.b, max(f.ca - R, 0), min(f.ca + R, f.ea - 1), max(f.cb - R, 0),
+                            min(f.cb + R, f.eb - 1))) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (k == kf) T[k] = D;
+                return true;
+            }
         }
     }
     // no valid point of the face strictly on the far side of F, visiting
     // only the far-side interval of each row (orient2(A, B, p) is affine in
     // p), within kHullScanWork rows and points
     if (!far_pt) {
-        const LPt2 o0 = {0, 0, -1}, eu = {1, 0, -1}, ev = {0, 1, -1};
+        const LPt2 o0 = {0, 0, 0}, eu = {1, 0, 0}, ev = {0, 1, 0};
         const int64_t d = orient2(A, B, o0);
         const int64_t nu = orient2(A, B, eu) - d, nv = orient2(A, B, ev) - d;
         const int64_t sg = sf > 0 ? 1 : -1;
         const int64_t budget = kHullScanWork / 32;
         int64_t work = 0;
         bool stop = false;
-        for (int64_t vv = lane; vv < ext[b] && !stop; vv += 32) {
+        for (int64_t vv = lane; vv < f.eb && !stop; vv += 32) {
             if (++work > budget) { stop = true; break; }
             int64_t t0, t1;
-            if (!positive_range(sg * nu, sg * (nv * (vv - c[b]) + d), -c[a], ext[a] - 1 - c[a], t0, t1)) continue;
+            if (!positive_range(sg * nu, sg * (nv * (vv - f.cb) + d), -(int64_t)f.ca, (int64_t)f.ea - 1 - f.ca, t0, t1))
+                continue;
             for (int64_t t = t0; t <= t1; ++t) {
-                int64_t pc[3] = {c[0], c[1], c[2]};
-                pc[a] = t + c[a];
-                pc[b] = vv;
-                if (++work > budget || valid[lattice_rank(S, pc[0], pc[1], pc[2])]) { stop = true; break; }
+                if (++work > budget || valid[f.rq + t * f.sa + (vv - f.cb) * f.sb]) { stop = true; break; }
             }
         }
         if (__any_sync(kAll, stop)) return false;
-        T[kf] = A;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k == kf) T[k] = A;
         return true;
     }
     return false;
@@ -921,53 +1024,73 @@ __device__ __forceinline__ int circle_fits_clearly(const float (&ctr)[2], float 
     return fit;
 }
 
-// The walk of `walk` on the face through c whose free axes are a < b: the
-// window is the square of radius R around c on that face, its points in
-// rank order (axis a fastest), shared out point by point. Returns 1 with the
-// triangle and q's barycentric coordinates, or 0.
-__device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], int a, int b,
+// The walk of `walk` on a face: the window is the square of radius R around
+// the entry, a row of it to each lane. Returns 1 with the triangle and q's
+// barycentric coordinates, or 0.
+__device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, const int64_t (&c)[3], const Face &f,
                                      int R, bool &settled, LPt2 (&T)[3], double (&lam)[3]) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, dv = lane - kMaxWindow2;
     const int64_t P = (int64_t)S.x * S.y * S.z;
-    const LPt2 q0 = {0, 0, -1};
-    // a is 0 or 1, b is 1 or 2
-    const int ca = (int)(a == 0 ? c[0] : c[1]), cb = (int)(b == 1 ? c[1] : c[2]);
-    const int ea = a == 0 ? S.x : S.y, eb = b == 1 ? S.y : S.z;
-    const int sa = a == 0 ? 1 : S.x, sb = b == 1 ? S.x : S.x * S.y;   // rank steps of the free axes
-    const int rq = (int)lattice_rank(S, c[0], c[1], c[2]);
-    const int u0 = max(ca - R, 0), u1 = min(ca + R, ea - 1), v0 = max(cb - R, 0), v1 = min(cb + R, eb - 1);
-    const int wu = u1 - u0 + 1, W = wu * (v1 - v0 + 1);
+    const LPt2 q0 = {0, 0, 0};
+    const int u0 = max(f.ca - R, 0), u1 = min(f.ca + R, f.ea - 1), v0 = max(f.cb - R, 0), v1 = min(f.cb + R, f.eb - 1);
+    const uint32_t row = face_row(f, R);
+    const uint32_t rim = abs(dv) < R ? (1u << (kMaxWindow2 - R)) | (1u << (kMaxWindow2 + R)) : ~0u;
+    const int r0 = f.rq + dv * f.sb - kMaxWindow2 * f.sa;   // the rank of bit k is r0 + k sa
     for (int it = 0; it < kMaxPivots; ++it) {
         float fc[2], fr2e;
         circumcircle_f(T, fc, fr2e);
-        const float fc0 = fc[0], fc1 = fc[1];
-        const float fr2 = fr2e * (1.0f + 1e-4f) + 1e-2f;   // as in walk
+        const float fc0 = fc[0], fv = (float)dv - fc[1];
+        const float margin = fr2e * 8e-6f + 1e-3f, fr2 = fr2e + margin;   // as in walk
         const bool deep = it < kDeepPivots;   // the pivot rule of walk
-        const bool shell = settled && it == 0;
+        const uint32_t m = settled && it == 0 ? row & rim : row;
+        const int split = (int)fminf(fmaxf(floorf(fc0), -(float)(kMaxWindow2 + 1)), (float)kMaxWindow2) + kMaxWindow2;
+        const uint32_t lowbits = split < 0 ? 0u : (2u << split) - 1u;
         int64_t best = kNone;
-        unsigned long long bkey = 0;
-        for (WinIter w(wu, 1 << 30, lane); w.k < W; w.step()) {
-            const int du = u0 + w.x - ca, dv = v0 + w.y - cb;
-            if (shell && max(abs(du), abs(dv)) < R) continue;
-            const int r = rq + du * sa + dv * sb;
-            if (!valid[r]) continue;
-            const float fu = (float)du - fc0, fv = (float)dv - fc1;
-            const float d2 = fu * fu + fv * fv;
-            if (d2 > fr2) continue;
-            if (T[0].rank == r || T[1].rank == r || T[2].rank == r) continue;
-            const LPt2 cand = {du, dv, r};
-            if (deep) {
-                const unsigned long long key = depth_key(fr2e - d2, r);
-                if (key > bkey && lifted_sign2(T, cand) > 0) bkey = key;
-            } else if (lifted_sign2(T, cand) > 0) {
-                best = r;
-                break;
+        unsigned bhi = 0, blo = 0;
+        auto scan = [&](bool exact) {
+#pragma unroll
+            for (int dir = 0; dir < 2; ++dir) {
+                uint32_t w = dir ? m & ~lowbits : m & lowbits;
+                while (w) {
+                    const int k = dir ? __ffs(w) - 1 : 31 - __clz(w);
+                    w &= ~(1u << k);
+                    const float fu = (float)(k - kMaxWindow2) - fc0;
+                    const float d2 = sum2(fu, fv);
+                    const int r = r0 + k * f.sa;
+                    const unsigned long long key = depth_key(fr2e - d2, r);
+                    const unsigned khi = (unsigned)(key >> 32), klo = (unsigned)key;
+                    if (khi < bhi) break;
+                    if (exact && d2 > fr2) break;
+                    if (khi == bhi && klo <= blo) continue;
+                    if (exact) {
+                        if (T[0].rank == (uint32_t)r || T[1].rank == (uint32_t)r || T[2].rank == (uint32_t)r) continue;
+                        const LPt2 cand = {k - kMaxWindow2, dv, (uint32_t)r};
+                        if (lifted_sign2(T, cand) <= 0) continue;
+                    }
+                    bhi = khi;
+                    blo = klo;
+                }
             }
-        }
+        };
         if (deep) {
-            bkey = warp_max_u64(bkey);
-            best = bkey ? (int64_t)(0xffffffffu - (unsigned)(bkey & 0xffffffffu)) : kNone;
+            scan(false);
+            const unsigned sure = __reduce_max_sync(kAll, bhi);
+            if (!(sure != 0 && depth_of(sure) > margin)) {
+                bhi = blo = 0;
+                scan(true);
+            }
+            const unsigned hi = __reduce_max_sync(kAll, bhi);
+            const unsigned lo = __reduce_max_sync(kAll, bhi == hi ? blo : 0u);
+            best = hi ? (int64_t)(0xffffffffu - lo) : kNone;
         } else {
+            for (uint32_t w = m; w && best == kNone; w &= w - 1) {
+                const int k = __ffs(w) - 1;
+                const float fu = (float)(k - kMaxWindow2) - fc0;
+                const int r = r0 + k * f.sa;
+                if (sum2(fu, fv) > fr2 || T[0].rank == (uint32_t)r || T[1].rank == (uint32_t)r || T[2].rank == (uint32_t)r) continue;
+                const LPt2 cand = {k - kMaxWindow2, dv, (uint32_t)r};
+                if (lifted_sign2(T, cand) > 0) best = r;
+            }
             best = warp_min(best);
         }
         const int64_t o = orient2(T[0], T[1], T[2]);   // > 0: T is kept counter-clockwise
@@ -980,17 +1103,17 @@ __device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, 
                 LPt2 u[3] = {T[0], T[1], T[2]};
                 u[k] = q0;
                 ol[k] = orient2(u[0], u[1], u[2]);
-                if (T[k].rank >= P) { ++nfar; kf = k; ofar = ol[k]; }
+                if (T[k].rank >= (uint32_t)P) { ++nfar; kf = k; ofar = ol[k]; }
             }
             const LPt2 t3[3] = {T[0], T[1], T[2]};   // the copies keep T itself in registers
             if (nfar == 0) {
-                const int fit = circle_fits_clearly(fc, fr2e, u0 - ca, u1 - ca, v0 - cb, v1 - cb, u0 > 0, u1 < ea - 1,
-                                                    v0 > 0, v1 < eb - 1);
+                const int fit = circle_fits_clearly(fc, fr2e, u0 - f.ca, u1 - f.ca, v0 - f.cb, v1 - f.cb, u0 > 0,
+                                                    u1 < f.ea - 1, v0 > 0, v1 < f.eb - 1);
                 if (fit == 0) return 0;
                 if (fit < 0) {
                     double ctr[2], r2;
                     circumcircle(t3, ctr, r2);
-                    if (!circle_fits(ctr, r2, S, c, a, b, u0, u1, v0, v1)) return 0;
+                    if (!circle_fits(ctr, r2, S, c, f.a, f.b, u0, u1, v0, v1)) return 0;
                 }
             } else if (nfar > 1 || ofar != 0) {
                 return 0;
@@ -999,7 +1122,7 @@ __device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, 
             for (int k = 0; k < 3; ++k) lam[k] = (double)ol[k] / (double)o;
             if (nfar == 0) return 1;
             LPt2 x3[3] = {T[0], T[1], T[2]};
-            if (!across_edge(S, valid, c, a, b, u0, u1, v0, v1, x3, kf)) return 0;
+            if (!across_edge(S, valid, c, f, R, x3, kf)) return 0;
 #pragma unroll
             for (int k = 0; k < 3; ++k) T[k] = x3[k];
             return 1;
@@ -1007,9 +1130,10 @@ __device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, 
         settled = false;
         int64_t bc[3];
         rank_coords(S, best, bc);
-        const LPt2 e = {(int32_t)(a == 0 ? bc[0] : bc[1]) - ca, (int32_t)(b == 1 ? bc[1] : bc[2]) - cb, best};
+        const LPt2 e = {(int32_t)(f.a == 0 ? bc[0] : bc[1]) - f.ca, (int32_t)(f.b == 1 ? bc[1] : bc[2]) - f.cb, (uint32_t)best};
         int leave = -1;
-        int64_t bq = 0, be = 0, brank = 0;
+        int64_t bq = 0, be = 0;
+            uint32_t brank = 0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             LPt2 u[3] = {T[0], T[1], T[2]};
@@ -1097,13 +1221,19 @@ constexpr int kTileN = kTileX * kTileY * kTileZ;
 // collects its missing interior entries, gathers the valid flags around the
 // tile into shared words, and its warps then take the collected entries one
 // at a time as they become free, all lanes on each. There are many more
-// tiles than CTAs fit on the chip, and the hardware hands them out, so the
-// tiles inside a missing slab (256 entries) and those with none even out.
-// Bound by dependent integer chains of the pivots. A 128^3 lattice with
-// 137,210 missing entries (88,000 of them here), the whole fill: 61 ms with
-// byte-wise window scans and one 32-entry chunk to a warp, 20 ms with the row
-// words, 12 ms with the pivots' determinants and ratio test shared out too.
-__global__ void __launch_bounds__(kFillThreads) fill_interior_kernel(int3 S, int tx, int ty,
+// tiles than CTAs fit on the chip, and the hardware hands them out, so those
+// inside a missing slab and those with nothing missing even out; the tile is
+// small because a slab's tile is what its four warps work through alone (8 x
+// 4 x 2: 6.5 ms, 16 x 4 x 4: a millisecond more again).
+// Bound by instructions: about 1,400 a pivot, a straight run of code far
+// longer than the instruction caches hold (most stalls are instruction
+// fetch), 16 pivots an entry. A 128^3 lattice with 137,210 missing entries
+// (88,000 of them here), the whole fill: 61 ms with byte-wise window scans
+// and one 32-entry chunk to a warp, 20 ms with the row words, 12 ms with the
+// pivots' determinants and ratio test shared out, 5.8 ms with the certain
+// pivots taken from the rows' nearest points, 32-bit minors, the row words in
+// the facet test and the faces, and this tile (5.2 here, 0.6 the boundary).
+__global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, int tx, int ty,
                                                                      const float *__restrict__ ends,
                                                                      const uint8_t *__restrict__ valid,
                                                                      float *__restrict__ out,
@@ -1155,6 +1285,7 @@ __global__ void __launch_bounds__(kFillThreads) fill_interior_kernel(int3 S, int
         start_tetrahedron(P, T);
         int ok = 0;
         bool settled = false;
+#pragma unroll 1
         for (int R = 2; R <= kMaxWindow && !ok; ++R)
             ok = walk(S, valid, win, lx, cx0 + lx, cy0 + ly, cz0 + lz, R, settled, T, lam);
         const int64_t vtx[4] = {T[0].rank, T[1].rank, T[2].rank, T[3].rank};
@@ -1193,7 +1324,7 @@ __device__ __forceinline__ void boundary_point(int3 S, const Boundary &n, int64_
     c[0] = t / yi / zi ? S.x - 1 : 0;
 }
 
-constexpr int kBoundaryChunk = 8;
+constexpr int kBoundaryChunk = 1;
 
 // The missing boundary entries: each warp takes kBoundaryChunk boundary
 // points and solves the missing ones one after another, all lanes on each.
@@ -1214,7 +1345,7 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, con
         const bool fixed[3] = {c[0] == 0 || c[0] == S.x - 1, c[1] == 0 || c[1] == S.y - 1,
                                c[2] == 0 || c[2] == S.z - 1};
         const int nfix = (int)fixed[0] + (int)fixed[1] + (int)fixed[2];
-        int64_t vtx[4] = {-1, -1, -1, -1};
+        int64_t vtx[4] = {-1, -1, -1, 0};
         double lam[4] = {0.0, 0.0, 0.0, 0.0};
         int nv = 0, ok = 0;   // flat: no tetrahedra; three fixed axes: a corner
         if (!flat && nfix == 1) {
@@ -1222,8 +1353,9 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, con
             LPt2 T2[3];
             double l2[3];
             start_triangle(P, T2);
+            const Face f = face_of(S, valid, c, a, b);
             bool settled = false;
-            for (int R = 2; R <= kMaxWindow2 && !ok; ++R) ok = walk2(S, valid, c, a, b, R, settled, T2, l2);
+            for (int R = 2; R <= kMaxWindow2 && !ok; ++R) ok = walk2(S, valid, c, f, R, settled, T2, l2);
             for (int k = 0; k < 3; ++k) { vtx[k] = T2[k].rank; lam[k] = l2[k]; }
             nv = 3;
         } else if (!flat && nfix == 2) {
