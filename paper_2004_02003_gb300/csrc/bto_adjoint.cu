@@ -82,6 +82,10 @@ using namespace bto::dev;
 constexpr int kMaxBins = 16384;      // bins of the sort: one CTA scans them, 16 a thread
 constexpr int64_t kSortMin = 2048;   // fewer particles keep the caller's order
 constexpr int kThreads = 128;
+// Up to this many particles per SM the forward takes four lanes for each: on
+// 152 SMs 20,000 particles over 50 cycles (the whole FTLE call) 359 us with
+// one lane, 326 with four, 2,000 258 and 216; 50,000 434 and 503.
+constexpr int64_t kQuadPerSm = 256;
 constexpr int kChunk = 24;           // cycles whose positions a thread of the scatter kernel holds at a time
 
 struct Stage {
@@ -376,6 +380,57 @@ __device__ __forceinline__ float3 adj_step(const float *__restrict__ f, float *_
     }
     add_cell(gF, g, acc_node, acc);
     return lx;
+}
+
+// The same by four lanes per particle (rk4_step_quad).
+__global__ void __launch_bounds__(kThreads) tape_forward_quad_kernel(
+    const BlockDev *__restrict__ blk, const void *const *__restrict__ table, int32_t L, int32_t C, float dt, int64_t P,
+    float4 *__restrict__ ckpt, int32_t *__restrict__ exitc, const int32_t *__restrict__ perm, float *__restrict__ ends,
+    uint8_t *__restrict__ valid, int32_t *__restrict__ exit_out) {
+    const BlockDev &B = *blk;
+    const Geo g = load_geo(B);
+    const float3 s = make_float3(dt * B.inv_h[0], dt * B.inv_h[1], dt * B.inv_h[2]);
+    const int64_t i = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 2;
+    const int lane4 = threadIdx.x & 3;
+    __shared__ int touched[kThreads];
+    const uint32_t word = (uint32_t)__cvta_generic_to_shared(touched + threadIdx.x);
+    const bool have = i < P;
+    float3 x = make_float3(0.f, 0.f, 0.f), q;
+    int32_t e = 0;
+    if (have) {
+        const float4 r = ckpt[i];
+        x = make_float3(r.x, r.y, r.z);
+        e = exitc[i];
+    }
+    bool alive = have && e < 0;
+    int32_t left = C;   // cycles left in the segment
+    float4 *ck = ckpt + i;
+    const void *next = table[0];
+    for (int32_t c = 0; c < L && __any_sync(0xffffffffu, alive); ++c) {
+        const void *field = next;
+        if (left == 0) {
+            ck += P;
+            if (alive && lane4 == 0) *ck = make_float4(x.x, x.y, x.z, 0.f);
+            left = C;
+        }
+        --left;
+        if (c + 1 < L) next = table[c + 1];
+        if (rk4_step_quad<bto::LAYOUT_F3>(x, field, g, s, q, alive, Ahead{c + 1 < L ? next : nullptr, word}, nullptr)) {
+            alive = false;
+            e = c;
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!have) return;
+    const int64_t o = perm[i];
+    if (lane4 < 3) {
+        const float v = lane4 == 0 ? x.x : (lane4 == 1 ? x.y : x.z);
+        ends[3 * o + lane4] = fmaf(v, B.h[lane4], B.origin[lane4]);
+    } else {
+        exitc[i] = e;
+        valid[o] = e < 0 ? 1 : 0;
+        if (exit_out) exit_out[o] = e;
+    }
 }
 
 // dk = J dp, column by column.
@@ -732,9 +787,14 @@ bto_status bto_tape_forward(bto_tape *t, const float *d_seeds, const void *const
                                           t->perm);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        const int g1 = (int)seg_grid(t).x;
-        tape_forward_kernel<<<g1, kThreads, 0, s>>>(t->d_block, d_field_table, t->L, t->C, dt, t->P, t->ckpt, t->exitc,
-                                                    t->perm, d_ends, d_valid, d_exit_cycle);
+        if (t->P <= kQuadPerSm * t->sm_count)
+            tape_forward_quad_kernel<<<(unsigned)((4 * t->P + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+                t->d_block, d_field_table, t->L, t->C, dt, t->P, t->ckpt, t->exitc, t->perm, d_ends, d_valid,
+                d_exit_cycle);
+        else
+            tape_forward_kernel<<<seg_grid(t).x, kThreads, 0, s>>>(t->d_block, d_field_table, t->L, t->C, dt, t->P,
+                                                                   t->ckpt, t->exitc, t->perm, d_ends, d_valid,
+                                                                   d_exit_cycle);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_st(e);

@@ -242,6 +242,143 @@ __device__ __forceinline__ int rk4_step(float3 &x, const void *__restrict__ fiel
     return rk4_step_src(x, GlobalSrc<LAYOUT>{field, g.nnx, g.nnxy, g.nodes, err}, g, s, q);
 }
 
+// ---------------------------------------------------------------------------
+// Four lanes per particle, for lists too short to fill the chip with one. A
+// particle's quad shares its cell: lane q holds the x-edge of the node row
+// (b, c) = (q & 1, q >> 1), six values loaded by six requests instead of 24,
+// and the quad blends the edges along y and z by exchange. A warp then waits
+// for eight particles' cell changes instead of 32, and four times as many
+// warps hide each other's loads. Every operation is the one trilerp_packed
+// performs, so the results are bitwise the same; the lanes of a quad hold the
+// same position and take the same branches.
+// ---------------------------------------------------------------------------
+struct QuadCell {
+    uint32_t node;     // ~0u when empty
+    float p[3], d[3];  // value at a = 0 and difference to a = 1
+};
+
+template <int LAYOUT>
+__device__ __forceinline__ float3 sample_quad(QuadCell &C, const void *__restrict__ field, const Geo &g, bool on,
+                                              float x, float y, float z, int32_t *err) {
+    const int q = threadIdx.x & 3;
+    int ix, iy, iz;
+    float fx, fy, fz;
+    cell_coord(x, g.cmx, ix, fx);
+    cell_coord(y, g.cmy, iy, fy);
+    cell_coord(z, g.cmz, iz, fz);
+    const uint32_t node = (uint32_t)ix + g.nnx * (uint32_t)iy + g.nnxy * (uint32_t)iz;
+    if (on && node != C.node) {
+        uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
+        if (!BTO_IN_BOUNDS((uint64_t)nd + 1 < g.nodes, err)) nd = 0;
+        float e[6];
+        if (LAYOUT == LAYOUT_F4) {
+            const float4 *f = reinterpret_cast<const float4 *>(field) + nd;
+            const float4 a0 = __ldg(f), a1 = __ldg(f + 1);
+            e[0] = a0.x; e[1] = a0.y; e[2] = a0.z;
+            e[3] = a1.x; e[4] = a1.y; e[5] = a1.z;
+        } else {
+            const float *f = reinterpret_cast<const float *>(field) + 3ull * nd;
+#pragma unroll
+            for (int m = 0; m < 6; ++m) e[m] = __ldg(f + m);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            C.p[k] = e[k];
+            C.d[k] = e[3 + k] - e[k];
+        }
+        C.node = node;
+    }
+    float r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float a = fmaf(fx, C.d[k], C.p[k]);
+        const float b = __shfl_xor_sync(0xffffffffu, a, 1);
+        const float y0 = (q & 1) ? b : a, y1 = (q & 1) ? a : b;
+        const float c = fmaf(fy, y1 - y0, y0);
+        const float d = __shfl_xor_sync(0xffffffffu, c, 2);
+        const float z0 = (q & 2) ? d : c, z1 = (q & 2) ? c : d;
+        r[k] = fmaf(fz, z1 - z0, z0);
+    }
+    return make_float3(r[0], r[1], r[2]);
+}
+
+// The cell of a point that may lie outside the closed box (clamped into it).
+__device__ __forceinline__ uint32_t near_cell(const Geo &g, float x, float y, float z) {
+    int i, j, k;
+    float f;
+    cell_coord(fminf(fmaxf(x, 0.f), g.fnx), g.cmx, i, f);
+    cell_coord(fminf(fmaxf(y, 0.f), g.fny), g.cmy, j, f);
+    cell_coord(fminf(fmaxf(z, 0.f), g.fnz), g.cmz, k, f);
+    return (uint32_t)i + g.nnx * (uint32_t)j + g.nnxy * (uint32_t)k;
+}
+
+// Brings the lane's node row of a cell into L1: asynchronous 4-byte copies of
+// its first and last word (the row spans up to two sectors) into a word of
+// shared memory that nobody reads. A plain load would hold a register and a
+// scoreboard; prefetch.global.L1 and .L2 measured half the gain and none.
+template <int LAYOUT>
+__device__ __forceinline__ void touch_row(const void *__restrict__ field, const Geo &g, uint32_t node, uint32_t word) {
+    constexpr uint32_t kNode = LAYOUT == LAYOUT_F4 ? 16 : 12;
+    const int q = threadIdx.x & 3;
+    const uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
+    const char *p = reinterpret_cast<const char *>(field) + (uint64_t)kNode * nd;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(word), "l"(p) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(word), "l"(p + 2 * kNode - 4) : "memory");
+}
+
+// What the quad's lookahead needs: the next cycle's field (NULL after the
+// last) and the shared word the touches go to.
+struct Ahead {
+    const void *next;
+    uint32_t word;
+};
+
+// rk4_step by a quad: all lanes of the warp call it; those with `on` false
+// load nothing and return 0 with x unchanged. Once k1 is known, the rows that
+// the step's last stage and the next step's first stages will most likely
+// sample are touched, so that their misses overlap stages 2 to 4.
+template <int LAYOUT>
+__device__ __forceinline__ int rk4_step_quad(float3 &x, const void *__restrict__ field, const Geo &g, const float3 s,
+                                             float3 &q, bool on, const Ahead ahead, int32_t *err) {
+    const float3 hs = make_float3(0.5f * s.x, 0.5f * s.y, 0.5f * s.z);
+    QuadCell C;
+    C.node = ~0u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) C.p[k] = C.d[k] = 0.f;
+    const bool start = on;
+    int failed = 0;
+    float px = x.x, py = x.y, pz = x.z;
+    float3 acc = make_float3(0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float3 v = sample_quad<LAYOUT>(C, field, g, on, px, py, pz, err);
+        if (k == 0 && on) {
+            const uint32_t n1 = near_cell(g, fmaf(s.x, v.x, x.x), fmaf(s.y, v.y, x.y), fmaf(s.z, v.z, x.z));
+            if (n1 != C.node) touch_row<LAYOUT>(field, g, n1, ahead.word);
+            if (ahead.next) {
+                touch_row<LAYOUT>(ahead.next, g, n1, ahead.word);
+                const uint32_t n2 = near_cell(g, fmaf(1.5f * s.x, v.x, x.x), fmaf(1.5f * s.y, v.y, x.y),
+                                              fmaf(1.5f * s.z, v.z, x.z));
+                if (n2 != n1) touch_row<LAYOUT>(ahead.next, g, n2, ahead.word);
+            }
+        }
+        if (k == 0) acc = v;
+        else if (k == 3) { acc.x += v.x; acc.y += v.y; acc.z += v.z; }
+        else { acc.x = fmaf(2.f, v.x, acc.x); acc.y = fmaf(2.f, v.y, acc.y); acc.z = fmaf(2.f, v.z, acc.z); }
+        const float sx6 = s.x * (1.f / 6.f), sy6 = s.y * (1.f / 6.f), sz6 = s.z * (1.f / 6.f);
+        if (k < 2) { px = fmaf(hs.x, v.x, x.x); py = fmaf(hs.y, v.y, x.y); pz = fmaf(hs.z, v.z, x.z); }
+        else if (k == 2) { px = fmaf(s.x, v.x, x.x); py = fmaf(s.y, v.y, x.y); pz = fmaf(s.z, v.z, x.z); }
+        else { px = fmaf(sx6, acc.x, x.x); py = fmaf(sy6, acc.y, x.y); pz = fmaf(sz6, acc.z, x.z); }
+        if (on && !inside(g, px, py, pz)) {
+            q = make_float3(px, py, pz);
+            failed = k + 1;
+            on = false;
+        }
+    }
+    if (start && !failed) x = make_float3(px, py, pz);
+    return failed;
+}
+
 // Termination location (the paper's future work, Sec. 6): the chord from the
 // last in-block position x to the first point q found outside is clipped to
 // the block, t = largest value in [0, 1] with x + t (q - x) inside; the exit

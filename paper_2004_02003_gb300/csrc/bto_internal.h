@@ -219,8 +219,10 @@ struct TiledArgs {
 // Kernel launchers (bto_kernels.cu). Each returns cudaGetLastError().
 cudaError_t launch_advect(const AdvectArgs &a, int layout, int nt, int ppt, bool cap, int grid,
                           size_t dyn_smem, cudaStream_t s);
-// All `cycles` cycles in one launch; a.fields is the [cycles][nb] table.
-cudaError_t launch_interval(const AdvectArgs &a, int layout, int32_t cycles, int64_t slots, int group, cudaStream_t s);
+// All `cycles` cycles in one launch; a.fields is the [cycles][nb] table. quad:
+// four lanes per particle.
+cudaError_t launch_interval(const AdvectArgs &a, int layout, int32_t cycles, int64_t slots, int group, bool quad,
+                            cudaStream_t s);
 cudaError_t advect_occupancy(int layout, int nt, int ppt, bool cap, bool batched, size_t dyn_smem,
                              int *ctas_per_sm);
 // Tiled advection (bto_tiled.cu).

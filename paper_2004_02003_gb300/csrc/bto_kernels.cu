@@ -247,6 +247,69 @@ __global__ void __launch_bounds__(kRegionAlign, kIntervalCtas) interval_kernel(c
     if (warp == first && lane == 0) a.p.gcnt[grp] = total;
 }
 
+// The same by four lanes per particle (rk4_step_quad): a CTA is one group.
+template <int LAYOUT>
+__global__ void __launch_bounds__(4 * kRegionAlign) interval_quad_kernel(const AdvectArgs a, const int32_t cycles,
+                                                                         const int group) {
+    __shared__ int kept[kRegionAlign / 8];
+    __shared__ int touched[4 * kRegionAlign];
+    const uint32_t word = (uint32_t)__cvta_generic_to_shared(touched + threadIdx.x);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = threadIdx.x & 3;
+    const int64_t s0 = (int64_t)blockIdx.x * group;   // the group's first slot
+    const int k = threadIdx.x >> 2;                   // slot in the group
+    int cnt = a.p.gcnt[blockIdx.x];
+    if (!BTO_IN_BOUNDS(cnt >= 0 && cnt <= group, a.err)) cnt = 0;
+    const int b = a.gblock[s0 / kUnit];
+    const BlockDev &B = a.blocks[b];
+    const Geo g = load_geo(B);
+    const float3 s = make_float3(a.dt * B.inv_h[0], a.dt * B.inv_h[1], a.dt * B.inv_h[2]);
+    const float *rec = a.p.rec + part_at(s0 + k, 0);
+    bool alive = k < cnt;
+    float3 x = make_float3(0.f, 0.f, 0.f);
+    int32_t id = 0;
+    if (alive) {
+        x = make_float3(__ldcs(rec), __ldcs(rec + 32), __ldcs(rec + 64));
+        id = __float_as_int(__ldcs(rec + 96));
+        if (!BTO_IN_BOUNDS(id >= 0 && id < B.nseeds, a.err)) alive = false;
+    }
+    const void *const *entry = a.fields + b;
+    const void *next = *entry;
+    for (int32_t c = 0; c < cycles && __any_sync(kFull, alive); ++c) {
+        const void *field = next;
+        if (c + 1 < cycles) {
+            entry += a.nb;
+            next = *entry;
+        }
+        const float3 x0 = x;
+        float3 out;
+        const int failed = rk4_step_quad<LAYOUT>(x, field, g, s, out, alive,
+                                                 Ahead{c + 1 < cycles ? next : nullptr, word}, a.err);
+        if (failed) {
+            alive = false;
+            if (q == 0) {
+                const int64_t gid = B.base + id;
+                __stcs(a.term + gid, make_float4(x0.x, x0.y, x0.z, __int_as_float(c)));
+                if (a.clip) __stcs(a.clip + gid, make_float4(out.x, out.y, out.z, __int_as_float(failed)));
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // survivors to the front of the group, in order, a field to each lane of the quad
+    const unsigned m = __ballot_sync(kFull, alive && q == 0);
+    if (lane == 0) kept[warp] = __popc(m);
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int w = 0; w < group / 8; ++w) {
+        if (w < warp) before += kept[w];
+        total += kept[w];
+    }
+    if (alive) {
+        const float v = q == 0 ? x.x : (q == 1 ? x.y : (q == 2 ? x.z : __int_as_float(id)));
+        __stcs(a.p.rec + part_at(s0 + before + __popc(m & ((1u << (lane & ~3)) - 1u)), q), v);
+    }
+    if (threadIdx.x == 0) a.p.gcnt[blockIdx.x] = total;
+}
+
 // ---------------------------------------------------------------------------
 // K2: seeds. Slot i of block b's region holds the lattice point perm[base + m]
 // (m = i - slot_base; brick order of the lattice); positions are the exact
@@ -567,7 +630,16 @@ cudaError_t launch_advect(const AdvectArgs &a, int layout, int nt, int ppt, bool
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_interval(const AdvectArgs &a, int layout, int32_t cycles, int64_t slots, int group, cudaStream_t s) {
+cudaError_t launch_interval(const AdvectArgs &a, int layout, int32_t cycles, int64_t slots, int group, bool quad,
+                            cudaStream_t s) {
+    if (quad) {
+        const unsigned groups = (unsigned)(slots / group);
+        if (layout == LAYOUT_F4)
+            interval_quad_kernel<LAYOUT_F4><<<groups, 4 * group, 0, s>>>(a, cycles, group);
+        else
+            interval_quad_kernel<LAYOUT_F3><<<groups, 4 * group, 0, s>>>(a, cycles, group);
+        return cudaGetLastError();
+    }
     const unsigned grid = (unsigned)(slots / kRegionAlign);
     if (layout == LAYOUT_F4)
         interval_kernel<LAYOUT_F4><<<grid, kRegionAlign, 0, s>>>(a, cycles, group);
