@@ -67,7 +67,7 @@ struct bto_tape {
     BlockDev *d_block = nullptr;
     int32_t *exitc = nullptr;   // P exit cycle, -1 while valid
     int32_t *perm = nullptr;    // P: the caller's index of each particle in cell order
-    int32_t *bins = nullptr;    // 2 * kMaxBins: counts (zero between calls) and starts of the sort
+    int32_t *bins = nullptr;    // 2 * kMaxBins: counts and starts of the sort
     int bsh[3] = {0, 0, 0};     // log2 of a bin's cells per axis
     int bn[3] = {1, 1, 1};      // bins per axis
     const void *const *table = nullptr;
@@ -84,8 +84,9 @@ constexpr int64_t kSortMin = 2048;   // fewer particles keep the caller's order
 constexpr int kThreads = 128;
 // Up to this many particles per SM the forward takes four lanes for each: on
 // 152 SMs 20,000 particles over 50 cycles (the whole FTLE call) 359 us with
-// one lane, 326 with four, 2,000 258 and 216; 50,000 434 and 503.
-constexpr int64_t kQuadPerSm = 256;
+// one lane, 326 with four, 2,000 258 and 216; 50,000 434 and 503; the forward
+// of 32,768 over 200 cycles 419 and 432.
+constexpr int64_t kQuadPerSm = 132;
 constexpr int kChunk = 24;           // cycles whose positions a thread of the scatter kernel holds at a time
 
 struct Stage {
@@ -171,9 +172,9 @@ __global__ void tape_bin_kernel(const BlockDev *__restrict__ blk, int64_t P, con
     }
 }
 
-// Step 2, one CTA: exclusive sums of the counts; the counts are left zero
-// for the next call. 16-byte accesses: a thread's 16 bins are consecutive.
-__global__ void __launch_bounds__(1024) tape_scan_kernel(int4 *__restrict__ count, int4 *__restrict__ start) {
+// Step 2, one CTA: exclusive sums of the counts. 16-byte accesses: a thread's
+// 16 bins are consecutive.
+__global__ void __launch_bounds__(1024) tape_scan_kernel(const int4 *__restrict__ count, int4 *__restrict__ start) {
     __shared__ int32_t part[32];
     constexpr int kPer = kMaxBins / 4096;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -182,7 +183,6 @@ __global__ void __launch_bounds__(1024) tape_scan_kernel(int4 *__restrict__ coun
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
         v[k] = count[threadIdx.x * kPer + k];
-        count[threadIdx.x * kPer + k] = make_int4(0, 0, 0, 0);
         sum += v[k].x + v[k].y + v[k].z + v[k].w;
     }
     int32_t incl = sum;
@@ -216,6 +216,7 @@ __global__ void tape_init_kernel(const BlockDev *__restrict__ blk, int64_t P, co
         if (place) {
             const int2 pl = place[i];
             at = (int64_t)start[pl.x] + pl.y;
+            if (at >= P) continue;   // only when forwards of one tape overlap: wrong results, no stray write
         }
         x0[at] = x;
         exitc[at] = inside(g, x.x, x.y, x.z) ? -1 : 0;   // a start outside the block never moves
@@ -750,7 +751,7 @@ bto_status bto_tape_create(const int32_t extent_cells[3], const float origin[3],
     if (e == cudaSuccess) e = t->mem.get(&t->exitc, sizeof(int32_t) * P);
     if (e == cudaSuccess) e = t->mem.get(&t->perm, sizeof(int32_t) * P);
     if (e == cudaSuccess) e = t->mem.get(&t->bins, sizeof(int32_t) * 2 * kMaxBins);
-    if (e == cudaSuccess) e = cudaMemset(t->bins, 0, sizeof(int32_t) * 2 * kMaxBins);
+    if (e == cudaSuccess) e = cudaMemset(t->perm, 0, sizeof(int32_t) * P);
     if (e == cudaSuccess) e = cudaMemcpy(t->d_block, &t->B, sizeof(BlockDev), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
@@ -779,8 +780,10 @@ bto_status bto_tape_forward(bto_tape *t, const float *d_seeds, const void *const
     int2 *place = t->P >= kSortMin ? reinterpret_cast<int2 *>(t->mat) : nullptr;
     if (place) {
         const Bins bins = {{t->bsh[0], t->bsh[1], t->bsh[2]}, {t->bn[0], t->bn[1], t->bn[2]}};
+        const cudaError_t z = cudaMemsetAsync(t->bins, 0, sizeof(int32_t) * kMaxBins, s);
+        if (z != cudaSuccess) return cuda_st(z);
         tape_bin_kernel<<<grid, 256, 0, s>>>(t->d_block, t->P, d_seeds, bins, t->bins, place);
-        tape_scan_kernel<<<1, 1024, 0, s>>>(reinterpret_cast<int4 *>(t->bins),
+        tape_scan_kernel<<<1, 1024, 0, s>>>(reinterpret_cast<const int4 *>(t->bins),
                                             reinterpret_cast<int4 *>(t->bins + kMaxBins));
     }
     tape_init_kernel<<<grid, 256, 0, s>>>(t->d_block, t->P, d_seeds, t->bins + kMaxBins, place, t->ckpt, t->exitc,

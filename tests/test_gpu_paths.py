@@ -103,8 +103,8 @@ def test_interval_end_equals_allocation_free_interval(n, stride):
 
 # Particles are independent: their ends and seed gradients do not depend on
 # the others, so not on whether the list is sorted by cell (2048 on) or takes
-# four lanes per particle (up to 256 per SM).
-@pytest.mark.parametrize("P", [1, 33, 2047, 2048, 45001])
+# four lanes per particle (up to 132 per SM).
+@pytest.mark.parametrize("P", [1, 33, 2047, 2048, 20064, 20065, 45001])
 def test_tape_results_do_not_depend_on_the_number_of_particles(P):
     import torch
     n, L, dt = (24, 20, 17), 21, 0.02
