@@ -183,14 +183,17 @@ BTO_API bto_status bto_end_interval_ex(bto_ctx *ctx, float *d_seeds, float *d_en
                                        uint8_t *d_valid, int32_t *d_exit_cycle,
                                        float *d_exit_pos, float *d_exit_time, bto_stream stream);
 
-/* Capture the cycles of one interval of a context into a CUDA graph and
- * launch it on `stream`; later intervals relaunch the cached graph.
+/* All cycles of one interval of a context, on `stream`. Without tiling this
+ * is one kernel that carries every particle through the interval in registers
+ * (particles are independent, and all fields are resident); with tiling, a
+ * CUDA graph of one launch per cycle, cached and relaunched.
  *   d_field_table  DEVICE array of interval_cycles*nb device pointers,
  *                  entry c*nb + b = field of block b in cycle c; it must
- *                  stay valid (and its entries point at the fields) for as
- *                  long as the graph is relaunched
+ *                  stay valid (and its entries point at the fields) until the
+ *                  interval has completed, with tiling for as long as the
+ *                  graph is relaunched
  *   dt             step of every cycle
- * Equivalent to interval_cycles advect calls, but one graph launch.
+ * Equivalent to interval_cycles advect calls, with the same results.
  * Must be called at cycle 0; leaves the context at cycle interval_cycles. */
 BTO_API bto_status bto_launch_interval_graph(bto_ctx *ctx, const void *const *d_field_table,
                                      float dt, bto_stream stream);

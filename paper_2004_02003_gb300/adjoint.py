@@ -9,8 +9,7 @@ checkpointed discrete adjoint kernels of libbto and returns the gradients
 with respect to the seeds and to every cycle's node velocities. Only
 argument marshalling happens here; all arithmetic runs in libbto.
 
-``ftle(tape, seeds, fields, dt)`` returns the flow-map Jacobian (three
-reverse sweeps) and the finite-time Lyapunov exponent of every particle that
+``ftle(tape, seeds, fields, dt)`` returns the flow-map Jacobian and the finite-time Lyapunov exponent of every particle that
 stays in its block for the interval.
 """
 from __future__ import annotations
@@ -21,8 +20,9 @@ from . import bto
 
 
 class Tape:
-    """Owning handle of a libbto tape (one block, P particles, L cycles,
-    positions kept every ``checkpoint_every`` cycles)."""
+    """Owning handle of a libbto tape (one block, P particles, L cycles). The
+    tape keeps positions at the start of segments whose length follows from L
+    alone; ``checkpoint_every`` is checked and otherwise without effect."""
 
     def __init__(self, extent, origin, spacing, num_particles, cycles, checkpoint_every=16):
         self.handle = bto.bto_tape_create(extent, origin, spacing, num_particles, cycles, checkpoint_every)
