@@ -493,7 +493,7 @@ def run_ours(args):
         "paper_metric_value": float(psteps) / cycles_s if cycles_s > 0 else None,
         "interval_end_ms": end_s * 1e3,
         "terminated_frac": float(1.0 - valid_np.mean()),
-        "gpu_launches": args.steps * (L + 3),
+        "gpu_launches": args.steps * (L + (3 if args.tile else 1)),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": frac,
                      "traffic": traffic, "peak_source": peak_src,
                      "algorithmic_bytes_per_launch": float(algo.mean()),
@@ -593,7 +593,7 @@ def extras(args, ctx, fields, gfields, table, out, exit_ref, psteps, dt, dev, st
     for p in plain:
         p.check(); p.close()
 
-    # (2) graph: the interval's cycles as one CUDA graph
+    # (2) graph: the interval's cycles in one call (one launch without tiling)
     g = bto.Context.batch(ext, org, spc, [STRIDE] * nb, L)
     g.set_layout(ctx_layout(args))
     g.set_launch(shape["threads_per_cta"], shape["particles_per_thread"], 0, shape["reg_cap"])
