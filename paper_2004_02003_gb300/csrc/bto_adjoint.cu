@@ -87,7 +87,11 @@ constexpr int kThreads = 128;
 // one lane, 326 with four, 2,000 258 and 216; 50,000 434 and 503; the forward
 // of 32,768 over 200 cycles 419 and 432.
 constexpr int64_t kQuadPerSm = 132;
-constexpr int kChunk = 24;           // cycles whose positions a thread of the scatter kernel holds at a time
+// Positions a thread of the scatter kernel holds: of up to kChunk consecutive
+// cycles and, in segments longer than that, of up to kSubs cycles spaced over
+// the segment to restart from (48 KB a CTA together).
+constexpr int kChunk = 24;
+constexpr int kSubs = 8;
 
 struct Stage {
     int ix, iy, iz;
@@ -570,10 +574,18 @@ __global__ void tape_product_kernel(const BlockDev *__restrict__ blk, int32_t L,
     }
 }
 
+// Cycles between the positions a long segment is restarted from: a multiple
+// of kChunk, at most kSubs of them.
+__host__ __device__ inline int32_t sub_space(int32_t C) {
+    return kChunk * ((C - 1) / (kChunk * kSubs) + 1);
+}
+
 // Field gradients of all segments: thread (s, i) takes the adjoint at the
 // end of segment s from the chain, recomputes the segment's positions from
-// its checkpoint into shared memory (kChunk cycles at a time, the last ones
-// first, in segments longer than that) and reverses its cycles.
+// its checkpoint into shared memory and reverses its cycles. A segment longer
+// than kChunk cycles (intervals over 400 cycles) is taken in chunks, the last
+// first; the first pass through it leaves a position every `space` cycles, and
+// the other chunks are recomputed from those.
 __global__ void __launch_bounds__(kThreads) tape_scatter_kernel(const BlockDev *__restrict__ blk,
                                                                 const void *const *__restrict__ table,
                                                                 float *const *__restrict__ gtable, int32_t L,
@@ -581,13 +593,15 @@ __global__ void __launch_bounds__(kThreads) tape_scatter_kernel(const BlockDev *
                                                                 const float4 *__restrict__ ckpt,
                                                                 const int32_t *__restrict__ exitc,
                                                                 const float *__restrict__ lam) {
-    extern __shared__ float pos[];   // [min(C, kChunk)][3][kThreads]
+    extern __shared__ float pos[];   // [min(C, kChunk) + positions to restart from][3][kThreads]
     const BlockDev &B = *blk;
     const Geo g = load_geo(B);
     const float3 s = make_float3(dt * B.inv_h[0], dt * B.inv_h[1], dt * B.inv_h[2]);
     const int32_t sg = blockIdx.y;
     const int32_t c0 = sg * C;
     float *mine = pos + threadIdx.x;
+    float *subs = mine + kChunk * 3 * kThreads;   // only in segments longer than kChunk
+    const int32_t space = sub_space(C);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t moved = cycles_moved(exitc[i], L);
         if (moved <= c0) continue;
@@ -597,9 +611,20 @@ __global__ void __launch_bounds__(kThreads) tape_scatter_kernel(const BlockDev *
         float3 lm = make_float3(l[0], l[(size_t)P], l[(size_t)2 * P]);
         for (int32_t k0 = c0 + (c1 - c0 - 1) / kChunk * kChunk, k1 = c1; k0 >= c0; k1 = k0, k0 -= kChunk) {
             float3 x = make_float3(r.x, r.y, r.z), q;
-            for (int32_t c = c0; c < k1; ++c) {
+            int32_t from = c0;
+            if (k1 < c1) {
+                const int32_t at = (k0 - c0) / space;
+                const float *m = subs + at * 3 * kThreads;
+                x = make_float3(m[0], m[kThreads], m[2 * kThreads]);
+                from = c0 + at * space;
+            }
+            for (int32_t c = from; c < k1; ++c) {
                 if (c >= k0) {
                     float *m = mine + (c - k0) * 3 * kThreads;
+                    m[0] = x.x; m[kThreads] = x.y; m[2 * kThreads] = x.z;
+                }
+                if (C > kChunk && k1 == c1 && (c - c0) % space == 0) {
+                    float *m = subs + (c - c0) / space * 3 * kThreads;
                     m[0] = x.x; m[kThreads] = x.y; m[2 * kThreads] = x.z;
                 }
                 if (c + 1 < k1) rk4_step<bto::LAYOUT_F3>(x, table[c], g, s, q);
@@ -819,7 +844,8 @@ bto_status bto_tape_backward(bto_tape *t, const float *d_grad_ends, float *d_gra
     tape_chain_kernel<<<grid, 256, 0, s>>>(t->d_block, t->L, t->C, t->P, t->exitc, t->perm, d_grad_ends,
                                            t->mat, d_grad_seeds);
     if (d_grad_field_table) {
-        const size_t smem = sizeof(float) * 3 * kThreads * (size_t)std::min(t->C, kChunk);
+        const int held = t->C <= kChunk ? t->C : kChunk + (t->C - 1) / sub_space(t->C) + 1;
+        const size_t smem = sizeof(float) * 3 * kThreads * (size_t)held;
         tape_scatter_kernel<<<seg_grid(t), kThreads, smem, s>>>(t->d_block, t->table, d_grad_field_table, t->L, t->C,
                                                                t->dt, t->P, t->ckpt, t->exitc, t->mat);
     }
