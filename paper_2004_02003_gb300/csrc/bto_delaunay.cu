@@ -248,10 +248,9 @@ __device__ __forceinline__ int fits_clearly(const float (&ctr)[3], float r2, int
 
 // Every routine from here on is warp-cooperative: the 32 lanes of a warp
 // solve one missing entry together. They hold the same simplex, split the
-// window's points between them (point k of the window goes to lane k mod
-// 32, k in rank order), and combine their findings with warp reductions,
-// so every decision is warp-uniform and equal to that of a serial scan in
-// rank order.
+// window's rows between them, and combine their findings with warp
+// reductions, so every decision is warp-uniform and equal to that of a serial
+// scan in rank order.
 constexpr unsigned kAll = 0xffffffffu;
 constexpr int64_t kNone = INT64_MAX;
 
