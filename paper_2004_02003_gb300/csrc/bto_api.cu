@@ -992,6 +992,10 @@ bto_status bto_autotune(bto_ctx *ctx, const void *const *d_field_table, int32_t 
     }
     const bto_status st2 = configure_launch(ctx);
     drop_graph(ctx);
+    // The trials' termination records go too: the interval's end takes a
+    // record of the cleared list for a particle that left in this interval.
+    ce = cudaMemsetAsync(ctx->term, 0xff, sizeof(float4) * (size_t)ctx->P, s);
+    if (ce != cudaSuccess) { (void)cudaGetLastError(); if (st == BTO_OK) st = cuda_status(ce); }
     const bto_status st3 = seed(ctx, s);
     BTO_CUDA(cudaStreamSynchronize(s));
     if (st != BTO_OK) return st;
