@@ -105,13 +105,23 @@ struct JCell {
     float v[8][3];
 };
 
-// Trilinear value, its Jacobian d v / d xi (cell units) and the cell, for a
-// point of the closed box.
+// cell_coord for any point, NaN and infinities included: the index is clamped
+// at both ends. A backward call retraces the forward's points, which are in
+// the box, only while the fields hold what they held then; where they have
+// been written since, its points may lie anywhere, and the nodes it reads and
+// adds to still are the block's.
+__device__ __forceinline__ void cell_coord_any(float x, float cm, int &i, float &f) {
+    const float t = fminf(fmaxf(__fadd_rd(x, 8388608.f), 8388608.f), cm);
+    i = __float_as_int(t) - 0x4B000000;
+    f = x - (t - 8388608.f);
+}
+
+// Trilinear value, its Jacobian d v / d xi (cell units) and the cell.
 __device__ __forceinline__ void sample_jac(JCell &C, const float *__restrict__ f, const Geo &g, float x, float y,
                                            float z, float3 &v, float (&J)[3][3], Stage &st) {
-    cell_coord(x, g.cmx, st.ix, st.fx);
-    cell_coord(y, g.cmy, st.iy, st.fy);
-    cell_coord(z, g.cmz, st.iz, st.fz);
+    cell_coord_any(x, g.cmx, st.ix, st.fx);
+    cell_coord_any(y, g.cmy, st.iy, st.fy);
+    cell_coord_any(z, g.cmz, st.iz, st.fz);
     const uint32_t node = (uint32_t)st.ix + g.nnx * (uint32_t)st.iy + g.nnxy * (uint32_t)st.iz;
     if (node != C.node) {
         load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, st.ix, st.iy, st.iz, C.v);
@@ -299,14 +309,14 @@ __device__ __forceinline__ void add_cell(float *__restrict__ gF, const Geo &g, u
     }
 }
 
-// The cell of x (a point of the closed box), its corners from the cache or
-// the field, and x's fractions in it.
+// The cell of x, its corners from the cache or the field, and x's fractions
+// in it.
 __device__ __forceinline__ void locate(JCell &C, const float *__restrict__ f, const Geo &g, const float3 x, float &fx,
                                        float &fy, float &fz) {
     int ix, iy, iz;
-    cell_coord(x.x, g.cmx, ix, fx);
-    cell_coord(x.y, g.cmy, iy, fy);
-    cell_coord(x.z, g.cmz, iz, fz);
+    cell_coord_any(x.x, g.cmx, ix, fx);
+    cell_coord_any(x.y, g.cmy, iy, fy);
+    cell_coord_any(x.z, g.cmz, iz, fz);
     const uint32_t node = (uint32_t)ix + g.nnx * (uint32_t)iy + g.nnxy * (uint32_t)iz;
     if (node != C.node) {
         load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, ix, iy, iz, C.v);
