@@ -390,8 +390,11 @@ __device__ __forceinline__ void store3(float *__restrict__ out, bool on, int64_t
 
 __global__ void __launch_bounds__(kRegionAlign) end_interval_kernel(const EndArgs a) {
     __shared__ float stage_all[kRegionAlign / 32][96];
+    // Launched programmatically itself (its launch overlaps the last cycle's
+    // tail); what follows it on the stream starts when it has completed, as
+    // after an ordinary launch: only the cycle calls let a caller's
+    // programmatic kernel start early.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float *stage = stage_all[threadIdx.x >> 5];
     const int64_t i = (int64_t)blockIdx.x * kRegionAlign + threadIdx.x;
     // the slot's record and its group's count do not wait for the block's geometry
