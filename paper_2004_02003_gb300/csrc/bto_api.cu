@@ -1094,7 +1094,10 @@ bto_status bto_fill_delaunay(const int32_t lattice[3], const float *d_ends, cons
         return BTO_ERR_INVALID_ARG;
     const int64_t P = (int64_t)lattice[0] * lattice[1] * lattice[2];
     if (P > (1ll << 31) - 1) return BTO_ERR_INVALID_ARG;
-    BTO_CUDA(bto::launch_fill_delaunay(lattice, d_ends, d_valid, d_out, d_status, (cudaStream_t)stream));
+    int dev = 0, sms = 0;
+    BTO_CUDA(cudaGetDevice(&dev));
+    BTO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    BTO_CUDA(bto::launch_fill_delaunay(lattice, d_ends, d_valid, d_out, d_status, sms, (cudaStream_t)stream));
     return BTO_OK;
 }
 

@@ -1213,17 +1213,125 @@ __device__ __forceinline__ void write_entry(int64_t P, int64_t p, bool ok, int n
 }
 
 constexpr int kFillThreads = 128;
+constexpr int kCopyTile = 4 * kFillThreads;   // entries of a CTA of the copy
+// Tiles for each CTA in flight from which on those with missing entries are
+// listed: below, the few waves of CTAs that find nothing cost no more than the
+// list's memset (33 x 31 x 29, none missing: 16 us either way). 64^3, none
+// missing: 14 us, 26 with a CTA to copy and look through each tile; 256^3: 89
+// and 1,310.
+constexpr int kListTiles = 4;
 constexpr int kTileN = kTileX * kTileY * kTileZ;
 
-// Copies the valid entries of the lattice (status 1) and solves the missing
-// interior ones. A CTA takes a tile: it copies the tile's valid entries and
-// collects its missing interior entries, gathers the valid flags around the
-// tile into shared words, and its warps then take the collected entries one
-// at a time as they become free, all lanes on each. There are many more
-// tiles than CTAs fit on the chip, and the hardware hands them out, so those
-// inside a missing slab and those with nothing missing even out; the tile is
-// small because a slab's tile is what its four warps work through alone (8 x
-// 4 x 2: 6.5 ms, 16 x 4 x 4: a millisecond more again).
+// How the solver's tiles are listed: groups of w tiles along x by v along z,
+// group (bx / w, by, bz / v) number bx / w + gx (by + ty (bz / v)).
+// w == 0: no list.
+struct Groups {
+    int tx, ty, tz;   // tiles per axis
+    int w, v;
+    int gx;           // groups along x
+};
+
+// Whether no interior entry of its group before (x, y, z), in lattice order,
+// is missing. Missing entries come in slabs: its neighbours first, then its
+// own row backward.
+__device__ __forceinline__ bool first_of_group(int3 S, const uint8_t *__restrict__ valid, const Groups &G, int x, int y,
+                                               int z) {
+    const int ex = kTileX * G.w, ez = kTileZ * G.v;
+    const int x0 = max(x / ex * ex, 1), x1 = min(x / ex * ex + ex, S.x - 1);   // x1 and y1: one past
+    const int y0 = max(y / kTileY * kTileY, 1), y1 = min(y / kTileY * kTileY + kTileY, S.y - 1);
+    const int z0 = max(z / ez * ez, 1);
+    const uint8_t *row = valid + lattice_rank(S, 0, y, z);
+    if ((y > y0 && !row[x - S.x]) || (z > z0 && !row[x - (int64_t)S.x * S.y])) return false;
+    for (int k = x - 1; k >= x0; --k)
+        if (!row[k]) return false;
+    for (int zz = z; zz >= z0; --zz)
+        for (int yy = (zz == z ? y : y1) - 1; yy >= y0; --yy) {
+            row = valid + lattice_rank(S, 0, yy, zz);
+            bool all = true;
+#pragma unroll 8
+            for (int k = x0; k < x1; ++k) all = all && row[k] != 0;
+            if (!all) return false;
+        }
+    return true;
+}
+
+// Copies the valid entries (status 1) and lists the groups that hold missing
+// interior entries, each by the first of them. The list stands in the out
+// entries of the plane z = 0, which are written last (by the boundary
+// kernel): word 0 counts the groups, word 1 the tiles the solver has taken,
+// the groups follow. On a lattice one point thick, which has no tetrahedra,
+// the missing entries are finished here. Bound by HBM: 16-byte accesses where
+// the pointers allow it.
+template <bool VEC>
+__global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const Groups G, bool flat,
+                                                                 const float *__restrict__ ends,
+                                                                 const uint8_t *__restrict__ valid,
+                                                                 float *__restrict__ out,
+                                                                 uint8_t *__restrict__ status) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the solver waits for this grid
+    const int64_t P = (int64_t)S.x * S.y * S.z, skip = G.w ? (int64_t)S.x * S.y : 0;
+    const int64_t t0 = (int64_t)blockIdx.x * kCopyTile;
+    unsigned miss = 0;   // bit k: the thread's entry k is missing
+    const bool vec = VEC && t0 >= skip && t0 + kCopyTile <= P;
+    if (vec) {
+        // ends and out 16-byte aligned, valid and status 4-byte: so is each tile
+        const uchar4 v4 = reinterpret_cast<const uchar4 *>(valid + t0)[threadIdx.x];
+        const uint8_t v[4] = {v4.x, v4.y, v4.z, v4.w};
+        uint8_t st[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            st[k] = v[k] ? 1 : 0;
+            miss |= v[k] ? 0u : 1u << k;
+        }
+        if (status) reinterpret_cast<uchar4 *>(status + t0)[threadIdx.x] = make_uchar4(st[0], st[1], st[2], st[3]);
+        const float4 *src = reinterpret_cast<const float4 *>(ends + 3 * t0);
+        float4 *dst = reinterpret_cast<float4 *>(out + 3 * t0);
+#pragma unroll
+        for (int k = 0; k < kCopyTile * 3 / 4 / kFillThreads; ++k)
+            dst[k * kFillThreads + threadIdx.x] = src[k * kFillThreads + threadIdx.x];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t p = t0 + k * kFillThreads + threadIdx.x;
+            if (p >= P) continue;
+            if (!valid[p]) {
+                miss |= 1u << k;
+                continue;
+            }
+            if (p >= skip) { out[3 * p] = ends[3 * p]; out[3 * p + 1] = ends[3 * p + 1]; out[3 * p + 2] = ends[3 * p + 2]; }
+            if (status) status[p] = 1;
+        }
+    }
+    if (flat) __syncthreads();   // the tile's copy before its missing entries' own values
+    if (!miss || !(flat || G.w)) return;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!(miss >> k & 1u)) continue;
+        const int64_t p = vec ? t0 + 4 * threadIdx.x + k : t0 + k * kFillThreads + threadIdx.x;
+        if (flat) {
+            const float nan = __int_as_float(0x7fc00000);
+            out[3 * p] = nan; out[3 * p + 1] = nan; out[3 * p + 2] = nan;
+            if (status) status[p] = 0;
+            continue;
+        }
+        const unsigned p32 = (unsigned)p, r = p32 / (unsigned)S.x;   // below 2^31
+        const int x = (int)(p32 - r * (unsigned)S.x), y = (int)(r % (unsigned)S.y), z = (int)(r / (unsigned)S.y);
+        if (x < 1 || x >= S.x - 1 || y < 1 || y >= S.y - 1 || z < 1 || z >= S.z - 1) continue;
+        if (!first_of_group(S, valid, G, x, y, z)) continue;
+        unsigned *list = reinterpret_cast<unsigned *>(out);
+        list[2 + atomicAdd(list, 1u)] = (unsigned)(x / (kTileX * G.w) + G.gx * (y / kTileY + G.ty * (z / (kTileZ * G.v))));
+    }
+}
+
+// Solves the missing interior entries. A CTA takes a tile: it collects the
+// tile's missing interior entries, gathers the valid flags around it into
+// shared words, and its warps then take the collected entries one at a time
+// as they become free, all lanes on each. The tile is small because a slab's
+// tile is what its four warps work through alone (8 x 4 x 2: 6.5 ms where this
+// took 5.8, 16 x 4 x 4 a millisecond more again), and no smaller, since its
+// entries share the words (8 x 2 x 1: 5.36 ms where this took 5.14). LISTED: the CTAs in flight take the tiles of
+// the listed groups from a counter; else every tile has a CTA, and the
+// hardware hands them out.
 // Bound by instructions: about 1,400 a pivot, a straight run of code far
 // longer than the instruction caches hold (most stalls are instruction
 // fetch), 16 pivots an entry. A 128^3 lattice with 137,210 missing entries
@@ -1231,123 +1339,183 @@ constexpr int kTileN = kTileX * kTileY * kTileZ;
 // and one 32-entry chunk to a warp, 20 ms with the row words, 12 ms with the
 // pivots' determinants and ratio test shared out, 5.8 ms with the certain
 // pivots taken from the rows' nearest points, 32-bit minors, the row words in
-// the facet test and the faces, and this tile (5.2 here, 0.6 the boundary).
-__global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, int tx, int ty,
+// the facet test and the faces, and this tile.
+template <bool LISTED>
+__global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, const Groups G,
                                                                      const float *__restrict__ ends,
                                                                      const uint8_t *__restrict__ valid,
                                                                      float *__restrict__ out,
                                                                      uint8_t *__restrict__ status) {
     __shared__ uint32_t words[kRowsY * kRowsZ];
     __shared__ uint8_t list[kTileN];
-    __shared__ int count, next;
-    static_assert(kTileN <= 256, "an entry's place in its tile is one byte");
+    __shared__ int count, next, tile[3];
+    static_assert(kTileN <= 32, "an entry of the tile to a lane");
     const int64_t P = (int64_t)S.x * S.y * S.z;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int bx = (int)(blockIdx.x % tx), by = (int)(blockIdx.x / tx % ty), bz = (int)(blockIdx.x / tx / ty);
-    const int cx0 = bx * kTileX, cy0 = by * kTileY, cz0 = bz * kTileZ;
-    if (threadIdx.x == 0) { count = 0; next = 0; }
-    __syncthreads();
-    for (int k = threadIdx.x; k < kTileN; k += kFillThreads) {
-        const int x = cx0 + k % kTileX, y = cy0 + k / kTileX % kTileY, z = cz0 + k / (kTileX * kTileY);
-        if (x >= S.x || y >= S.y || z >= S.z) continue;
-        const int64_t p = lattice_rank(S, x, y, z);
-        if (valid[p]) {
-            out[3 * p] = ends[3 * p]; out[3 * p + 1] = ends[3 * p + 1]; out[3 * p + 2] = ends[3 * p + 2];
-            if (status) status[p] = 1;
-        } else if (x > 0 && x < S.x - 1 && y > 0 && y < S.y - 1 && z > 0 && z < S.z - 1) {
-            list[atomicAdd(&count, 1)] = (uint8_t)k;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    unsigned *listed = reinterpret_cast<unsigned *>(out);
+    const unsigned sub = (unsigned)(G.w * G.v), total = LISTED ? __ldcg(listed) * sub : 0u;
+#pragma unroll 1
+    for (;;) {
+        if (warp == 0) {
+            int bx, by, bz;
+            if (LISTED) {
+                unsigned job = 0, g = 0;
+                if (lane == 0) {
+                    job = atomicAdd(listed + 1, 1u);
+                    if (job < total) g = __ldcg(listed + 2 + job / sub);
+                }
+                job = __shfl_sync(kAll, job, 0);
+                g = __shfl_sync(kAll, g, 0);
+                const int in = (int)(job % sub);
+                bx = (int)(g % (unsigned)G.gx) * G.w + in % G.w;
+                by = (int)(g / (unsigned)G.gx % (unsigned)G.ty);
+                bz = (int)(g / (unsigned)G.gx / (unsigned)G.ty) * G.v + in / G.w;
+                if (job >= total) bx = -1;   // none left
+            } else {
+                bx = (int)(blockIdx.x % G.tx);
+                by = (int)(blockIdx.x / G.tx % G.ty);
+                bz = (int)(blockIdx.x / G.tx / G.ty);
+            }
+            const int x = bx * kTileX + lane % kTileX, y = by * kTileY + lane / kTileX % kTileY,
+                      z = bz * kTileZ + lane / (kTileX * kTileY);
+            bool missing = false;
+            if (lane < kTileN && x > 0 && x < S.x - 1 && y > 0 && y < S.y - 1 && z > 0 && z < S.z - 1)
+                missing = !valid[lattice_rank(S, x, y, z)];
+            const unsigned m = __ballot_sync(kAll, missing);
+            if (missing) list[__popc(m & ((1u << lane) - 1u))] = (uint8_t)lane;
+            if (lane == 0) {
+                count = __popc(m);
+                next = 0;
+                tile[0] = bx;
+                tile[1] = by;
+                tile[2] = bz;
+            }
         }
-    }
-    __syncthreads();
-    const int missing = count;
-    if (missing == 0) return;
-    const int gx = cx0 - kMaxWindow + lane;
+        __syncthreads();
+        if (LISTED && tile[0] < 0) return;
+        const int missing = count;
+        if (missing) {
+            const int cx0 = tile[0] * kTileX, cy0 = tile[1] * kTileY, cz0 = tile[2] * kTileZ;
+            const int gx = cx0 - kMaxWindow + lane;
 #pragma unroll 4
-    for (int row = warp; row < kRowsY * kRowsZ; row += kFillThreads / 32) {
-        const int y = cy0 - kMaxWindow + row % kRowsY, z = cz0 - kMaxWindow + row / kRowsY;
-        bool v = false;
-        if (gx >= 0 && gx < S.x && y >= 0 && y < S.y && z >= 0 && z < S.z) v = valid[lattice_rank(S, gx, y, z)] != 0;
-        const unsigned w = __ballot_sync(kAll, v);
-        if (lane == 0) words[row] = w;
+            for (int row = warp; row < kRowsY * kRowsZ; row += kFillThreads / 32) {
+                const int y = cy0 - kMaxWindow + row % kRowsY, z = cz0 - kMaxWindow + row / kRowsY;
+                bool v = false;
+                if (gx >= 0 && gx < S.x && y >= 0 && y < S.y && z >= 0 && z < S.z) v = valid[lattice_rank(S, gx, y, z)] != 0;
+                const unsigned w = __ballot_sync(kAll, v);
+                if (lane == 0) words[row] = w;
+            }
+            __syncthreads();
+            for (;;) {
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&next, 1);
+                at = __shfl_sync(kAll, at, 0);
+                if (at >= missing) break;
+                const int k = list[at];
+                const int lx = k % kTileX, ly = k / kTileX % kTileY, lz = k / (kTileX * kTileY);
+                const uint32_t *win = words + (ly + kMaxWindow) + kRowsY * (lz + kMaxWindow);
+                const volatile int *t = tile;   // read again for each entry: the walk needs the registers
+                const int cx = t[0] * kTileX + lx, cy = t[1] * kTileY + ly, cz = t[2] * kTileZ + lz;
+                LPt T[4];
+                double lam[4] = {0.0, 0.0, 0.0, 0.0};
+                start_tetrahedron(P, T);
+                int ok = 0;
+                bool settled = false;
+#pragma unroll 1
+                for (int R = 2; R <= kMaxWindow && !ok; ++R)
+                    ok = walk(S, valid, win, lx, cx, cy, cz, R, settled, T, lam);
+                const int64_t vtx[4] = {T[0].rank, T[1].rank, T[2].rank, T[3].rank};
+                write_entry(P, lattice_rank(S, cx, cy, cz), ok == 1, 4, vtx, lam, ends, out, status);
+            }
+        }
+        if (!LISTED) return;
+        __syncthreads();   // the tile's words and list are free again
+    }
+}
+
+// The lattice's boundary points (fewer than 2^31), numbered: the z faces, then
+// what the y faces, then what the x faces add.
+struct Boundary {
+    unsigned nz, ny, nx;
+};
+__host__ __device__ inline Boundary boundary_of(int3 S) {
+    const unsigned zi = S.z > 2 ? S.z - 2 : 0, yi = S.y > 2 ? S.y - 2 : 0;
+    return Boundary{(unsigned)S.x * S.y * (S.z > 1 ? 2 : 1), S.x * zi * (S.y > 1 ? 2 : 1), yi * zi * (S.x > 1 ? 2 : 1)};
+}
+__device__ __forceinline__ void boundary_point(int3 S, const Boundary &n, unsigned t, int (&c)[3]) {
+    const unsigned sx = S.x, zi = S.z - 2, yi = S.y - 2;
+    if (t < n.nz) {
+        const unsigned r = t / sx, top = r >= (unsigned)S.y;
+        c[0] = t - r * sx;
+        c[1] = top ? r - S.y : r;
+        c[2] = top ? S.z - 1 : 0;
+        return;
+    }
+    t -= n.nz;
+    if (t < n.ny) {
+        const unsigned r = t / sx, top = r >= zi;
+        c[0] = t - r * sx;
+        c[2] = 1 + (top ? r - zi : r);
+        c[1] = top ? S.y - 1 : 0;
+        return;
+    }
+    t -= n.ny;
+    const unsigned r = t / yi, top = r >= zi;
+    c[1] = 1 + t - r * yi;
+    c[2] = 1 + (top ? r - zi : r);
+    c[0] = top ? S.x - 1 : 0;
+}
+
+// The missing boundary entries: a CTA takes `points` boundary points (4 to
+// 128) and its warps solve the missing ones as they become free, all lanes on
+// each. Where the plane z = 0 has held the solver's list (`plane0`), its valid
+// entries are copied here.
+__global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, int points, bool plane0,
+                                                                     const float *__restrict__ ends,
+                                                                     const uint8_t *__restrict__ valid,
+                                                                     float *__restrict__ out,
+                                                                     uint8_t *__restrict__ status) {
+    __shared__ uint8_t list[kFillThreads];
+    __shared__ int count, next;
+    const int64_t P = (int64_t)S.x * S.y * S.z;
+    const Boundary n = boundary_of(S);
+    const unsigned total = n.nz + n.ny + n.nx, t0 = blockIdx.x * (unsigned)points;
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) count = next = 0;
+    // Waits for the solver. Started beside the solver's last tiles, on points
+    // off the list's plane, it made the whole fill 3% slower: two kernels that
+    // are bound by instruction fetch then share the caches.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+    if ((int)threadIdx.x < points && t0 + threadIdx.x < total) {
+        int c[3];
+        boundary_point(S, n, t0 + threadIdx.x, c);
+        const int64_t p = lattice_rank(S, c[0], c[1], c[2]);
+        if (!valid[p]) {
+            list[atomicAdd(&count, 1)] = (uint8_t)threadIdx.x;
+        } else if (plane0 && c[2] == 0) {
+            out[3 * p] = ends[3 * p]; out[3 * p + 1] = ends[3 * p + 1]; out[3 * p + 2] = ends[3 * p + 2];
+        }
     }
     __syncthreads();
     for (;;) {
         int at = 0;
         if (lane == 0) at = atomicAdd(&next, 1);
         at = __shfl_sync(kAll, at, 0);
-        if (at >= missing) break;
-        const int k = list[at];
-        const int lx = k % kTileX, ly = k / kTileX % kTileY, lz = k / (kTileX * kTileY);
-        const uint32_t *win = words + (ly + kMaxWindow) + kRowsY * (lz + kMaxWindow);
-        LPt T[4];
-        double lam[4] = {0.0, 0.0, 0.0, 0.0};
-        start_tetrahedron(P, T);
-        int ok = 0;
-        bool settled = false;
-#pragma unroll 1
-        for (int R = 2; R <= kMaxWindow && !ok; ++R)
-            ok = walk(S, valid, win, lx, cx0 + lx, cy0 + ly, cz0 + lz, R, settled, T, lam);
-        const int64_t vtx[4] = {T[0].rank, T[1].rank, T[2].rank, T[3].rank};
-        write_entry(P, lattice_rank(S, cx0 + lx, cy0 + ly, cz0 + lz), ok == 1, 4, vtx, lam, ends, out, status);
-    }
-}
-
-// The lattice's boundary points, numbered: the z faces, then what the y
-// faces, then what the x faces add.
-struct Boundary {
-    int64_t nz, ny, nx;
-};
-__host__ __device__ inline Boundary boundary_of(int3 S) {
-    const int64_t zi = S.z > 2 ? S.z - 2 : 0, yi = S.y > 2 ? S.y - 2 : 0;
-    return Boundary{(int64_t)S.x * S.y * (S.z > 1 ? 2 : 1), S.x * zi * (S.y > 1 ? 2 : 1), yi * zi * (S.x > 1 ? 2 : 1)};
-}
-__device__ __forceinline__ void boundary_point(int3 S, const Boundary &n, int64_t t, int64_t (&c)[3]) {
-    if (t < n.nz) {
-        c[0] = t % S.x;
-        c[1] = t / S.x % S.y;
-        c[2] = t / S.x / S.y ? S.z - 1 : 0;
-        return;
-    }
-    t -= n.nz;
-    const int64_t zi = S.z - 2;
-    if (t < n.ny) {
-        c[0] = t % S.x;
-        c[2] = 1 + t / S.x % zi;
-        c[1] = t / S.x / zi ? S.y - 1 : 0;
-        return;
-    }
-    t -= n.ny;
-    const int64_t yi = S.y - 2;
-    c[1] = 1 + t % yi;
-    c[2] = 1 + t / yi % zi;
-    c[0] = t / yi / zi ? S.x - 1 : 0;
-}
-
-constexpr int kBoundaryChunk = 1;
-
-// The missing boundary entries: each warp takes kBoundaryChunk boundary
-// points and solves the missing ones one after another, all lanes on each.
-__global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, const float *__restrict__ ends,
-                                                                     const uint8_t *__restrict__ valid,
-                                                                     float *__restrict__ out,
-                                                                     uint8_t *__restrict__ status) {
-    const int64_t P = (int64_t)S.x * S.y * S.z;
-    const Boundary n = boundary_of(S);
-    const int64_t total = n.nz + n.ny + n.nx;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const bool flat = S.x == 1 || S.y == 1 || S.z == 1;
-    for (int64_t t = warp * kBoundaryChunk; t < min((warp + 1) * kBoundaryChunk, total); ++t) {
-        int64_t c[3];
-        boundary_point(S, n, t, c);
+        if (at >= count) break;
+        int c32[3];
+        boundary_point(S, n, t0 + list[at], c32);
+        const int64_t c[3] = {c32[0], c32[1], c32[2]};
         const int64_t p = lattice_rank(S, c[0], c[1], c[2]);
-        if (valid[p]) continue;
         const bool fixed[3] = {c[0] == 0 || c[0] == S.x - 1, c[1] == 0 || c[1] == S.y - 1,
                                c[2] == 0 || c[2] == S.z - 1};
         const int nfix = (int)fixed[0] + (int)fixed[1] + (int)fixed[2];
         int64_t vtx[4] = {-1, -1, -1, 0};
         double lam[4] = {0.0, 0.0, 0.0, 0.0};
-        int nv = 0, ok = 0;   // flat: no tetrahedra; three fixed axes: a corner
-        if (!flat && nfix == 1) {
+        int nv = 0, ok = 0;   // three fixed axes: a corner
+        if (nfix == 1) {
             const int a = fixed[0] ? 1 : 0, b = fixed[2] ? 1 : 2;
             LPt2 T2[3];
             double l2[3];
@@ -1357,7 +1525,7 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, con
             for (int R = 2; R <= kMaxWindow2 && !ok; ++R) ok = walk2(S, valid, c, f, R, settled, T2, l2);
             for (int k = 0; k < 3; ++k) { vtx[k] = T2[k].rank; lam[k] = l2[k]; }
             nv = 3;
-        } else if (!flat && nfix == 2) {
+        } else if (nfix == 2) {
             const int a = !fixed[0] ? 0 : (!fixed[1] ? 1 : 2);
             ok = edge_interp(S, valid, c, a, vtx, lam);
             nv = 2;
@@ -1370,19 +1538,76 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, con
 
 BTO_BOUNDS_ACCESSOR(bounds_failures_delaunay)
 
+// The solver's groups, and whether their list fits the plane z = 0 of out.
+static Groups groups_of(const int32_t S[3], bool listed) {
+    Groups G{};
+    G.tx = (S[0] + kTileX - 1) / kTileX;
+    G.ty = (S[1] + kTileY - 1) / kTileY;
+    G.tz = (S[2] + kTileZ - 1) / kTileZ;
+    if (!listed) return G;
+    G.w = G.tx < 4 ? G.tx : 4;
+    G.gx = (G.tx + G.w - 1) / G.w;
+    const int64_t room = (3 * (int64_t)S[0] * S[1] - 2) / ((int64_t)G.gx * G.ty);   // groups along z: 1 or more
+    const int64_t gz = room < G.tz ? room : G.tz;
+    G.v = (int)((G.tz + gz - 1) / gz);
+    return G;
+}
+
+// A launch that may start once every CTA of the kernel before it has started.
+template <class... Params, class... Args>
+static cudaError_t launch_after(void (*kernel)(Params...), int64_t grid, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kFillThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 cudaError_t launch_fill_delaunay(const int32_t S[3], const float *ends, const uint8_t *valid, float *out,
-                                 uint8_t *status, cudaStream_t s) {
+                                 uint8_t *status, int sm_count, cudaStream_t s) {
     const int3 S3 = make_int3(S[0], S[1], S[2]);
-    const int64_t tx = (S[0] + kTileX - 1) / kTileX, ty = (S[1] + kTileY - 1) / kTileY, tz = (S[2] + kTileZ - 1) / kTileZ;
-    fill_interior_kernel<<<(unsigned)(tx * ty * tz), kFillThreads, 0, s>>>(S3, (int)tx, (int)ty, ends, valid, out,
-                                                                          status);
+    const int64_t P = (int64_t)S[0] * S[1] * S[2];
+    const bool flat = S[0] == 1 || S[1] == 1 || S[2] == 1;
+    const bool inner = S[0] > 2 && S[1] > 2 && S[2] > 2;
+    const int64_t tiles = (int64_t)((S[0] + kTileX - 1) / kTileX) * ((S[1] + kTileY - 1) / kTileY) * ((S[2] + kTileZ - 1) / kTileZ);
+    const int64_t resident = 4ll * sm_count;
+    const bool apart = out + 3 * P <= ends || ends + 3 * P <= out;   // the list would spoil ends
+    const bool listed = inner && apart && tiles > kListTiles * resident;
+    const Groups G = groups_of(S, listed);
+    if (listed) {
+        const cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+    }
+    const unsigned copies = (unsigned)((P + kCopyTile - 1) / kCopyTile);
+    const bool vec = !((reinterpret_cast<uintptr_t>(ends) | reinterpret_cast<uintptr_t>(out)) & 15u) &&
+                     !((reinterpret_cast<uintptr_t>(valid) | reinterpret_cast<uintptr_t>(status)) & 3u);
+    if (vec)
+        fill_copy_kernel<true><<<copies, kFillThreads, 0, s>>>(S3, G, flat, ends, valid, out, status);
+    else
+        fill_copy_kernel<false><<<copies, kFillThreads, 0, s>>>(S3, G, flat, ends, valid, out, status);
     cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || flat) return e;
+    if (listed)
+        e = launch_after(fill_interior_kernel<true>, resident, s, S3, G, ends, valid, out, status);
+    else if (inner)
+        e = launch_after(fill_interior_kernel<false>, tiles, s, S3, G, ends, valid, out, status);
     if (e != cudaSuccess) return e;
     const Boundary n = boundary_of(S3);
-    const int64_t per = kBoundaryChunk * (kFillThreads / 32);
-    fill_boundary_kernel<<<(unsigned)((n.nz + n.ny + n.nx + per - 1) / per), kFillThreads, 0, s>>>(S3, ends, valid, out,
-                                                                                              status);
-    return cudaGetLastError();
+    const int64_t total = (int64_t)n.nz + n.ny + n.nx;
+    // Points of a CTA: its warps share a run of missing ones, so few where
+    // those bound the call (40^3 with losses at every face: 348 us with 4, 396
+    // with 16; 128^3: 5.30 ms with 4, 5.34 with 8, 5.41 with 64), and more
+    // where the CTAs that find nothing do (none missing: 128^3 39 us with 4,
+    // 27 with 8, 20 with 16; 256^3 201, 138, 105, and 89 with 32).
+    int points = total <= 16 * resident ? 4 : 8;
+    while (points < kFillThreads && total > 32 * resident * points) points *= 2;
+    return launch_after(fill_boundary_kernel, (total + points - 1) / points, s, S3, points, listed, ends, valid, out,
+                        status);
 }
 
 }  // namespace bto
