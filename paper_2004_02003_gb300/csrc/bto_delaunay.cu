@@ -1329,9 +1329,9 @@ __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const G
 // as they become free, all lanes on each. The tile is small because a slab's
 // tile is what its four warps work through alone (8 x 4 x 2: 6.5 ms where this
 // took 5.8, 16 x 4 x 4 a millisecond more again), and no smaller, since its
-// entries share the words (8 x 2 x 1: 5.36 ms where this took 5.14). LISTED: the CTAs in flight take the tiles of
-// the listed groups from a counter; else every tile has a CTA, and the
-// hardware hands them out.
+// entries share the words (8 x 2 x 1: 5.36 ms where this took 5.14). LISTED:
+// the CTAs in flight take the tiles of the listed groups from a counter; else
+// every tile has a CTA, and the hardware hands them out.
 // Bound by instructions: about 1,400 a pivot, a straight run of code far
 // longer than the instruction caches hold (most stalls are instruction
 // fetch), 16 pivots an entry. A 128^3 lattice with 137,210 missing entries
