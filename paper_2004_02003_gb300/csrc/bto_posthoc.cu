@@ -84,10 +84,27 @@ __global__ void __launch_bounds__(kFillThreads) fill_lattice_kernel(int3 S, cons
         for (int k = 0; k < kFillTile * 3 / 4 / kFillThreads; ++k)
             dst[k * kFillThreads + threadIdx.x] = src[k * kFillThreads + threadIdx.x];
     } else {
-        for (int i = threadIdx.x; i < n; i += kFillThreads) {
+        // a small lattice waits for its last tile alone: the four entries of
+        // a thread are loaded together, the missing ones' ends for nothing
+        // (33 x 31 x 29: 10.9 us with one entry after another, 8.9 so)
+        constexpr int kPer = kFillTile / kFillThreads;
+        uint8_t v[kPer];
+        float e[kPer][3];
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int i = k * kFillThreads + threadIdx.x;
+            const int64_t p = t0 + (i < n ? i : 0);
+            v[k] = valid[p];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) e[k][d] = ends[3 * p + d];
+        }
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int i = k * kFillThreads + threadIdx.x;
             const int64_t p = t0 + i;
-            if (valid[p]) {
-                out[3 * p] = ends[3 * p]; out[3 * p + 1] = ends[3 * p + 1]; out[3 * p + 2] = ends[3 * p + 2];
+            if (i >= n) continue;
+            if (v[k]) {
+                out[3 * p] = e[k][0]; out[3 * p + 1] = e[k][1]; out[3 * p + 2] = e[k][2];
                 if (status) status[p] = 1;
             } else {
                 list[atomicAdd(&count, 1)] = (uint16_t)i;
