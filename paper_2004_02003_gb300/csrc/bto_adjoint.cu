@@ -80,7 +80,16 @@ namespace {
 using namespace bto::dev;
 
 constexpr int kMaxBins = 16384;      // bins of the sort: one CTA scans them, 16 a thread
-constexpr int64_t kSortMin = 2048;   // fewer particles keep the caller's order
+// Whether a forward sorts its particles. The sort costs 9 us and more with the
+// particles, and pays by every cycle after it, in the forward and in the
+// backward calls: never in one or two cycles (forward of 1M particles over 1:
+// 111 us sorted, 64 not; 20,000 over 2: 28 and 15), below 10 from about
+// 400,000 particle-cycles on (forward and field gradients of 60,000 over 8:
+// 140 and 156 us, 60,000 over 4: 95 and 99, the forward alone 38 and 27;
+// 200,000 over 4: 175 and 224), then in all but small calls.
+inline bool sorts(int64_t P, int32_t L) {
+    return L >= 10 ? P >= 2048 : L >= 3 && P * L >= 400000;
+}
 constexpr int kThreads = 128;
 // Up to this many particles per SM the forward takes four lanes for each: on
 // 152 SMs 20,000 particles over 50 cycles (the whole FTLE call) 359 us with
@@ -812,7 +821,7 @@ bto_status bto_tape_forward(bto_tape *t, const float *d_seeds, const void *const
     t->dt = dt;
     t->have_forward = false;
     // the sort's (bin, place) pairs use the matrices' memory, which a backward call writes afresh
-    int2 *place = t->P >= kSortMin ? reinterpret_cast<int2 *>(t->mat) : nullptr;
+    int2 *place = sorts(t->P, t->L) ? reinterpret_cast<int2 *>(t->mat) : nullptr;
     if (place) {
         const Bins bins = {{t->bsh[0], t->bsh[1], t->bsh[2]}, {t->bn[0], t->bn[1], t->bn[2]}};
         const cudaError_t z = cudaMemsetAsync(t->bins, 0, sizeof(int32_t) * kMaxBins, s);
