@@ -118,7 +118,10 @@ BTO_API bto_status bto_set_field_layout(bto_ctx *ctx, bto_field_layout layout);
  * Allocates 2 x (largest block's nodes) x 16 bytes on first use. Only at
  * cycle 0 and with the F3_AOS layout, else BTO_ERR_STATE; not available
  * with bto_launch_interval_graph (BTO_ERR_UNSUPPORTED). enable = 0 goes
- * back to gathering from the caller's F3 field directly (the default). */
+ * back to gathering from the caller's F3 field directly (the default). Each
+ * launch then holds one block, so a launch shape that neither bto_set_launch
+ * nor bto_autotune has set follows the largest block while ingest is on; a
+ * change of particles per thread reseeds the interval (synchronously). */
 BTO_API bto_status bto_set_ingest(bto_ctx *ctx, int32_t enable);
 
 /* Total number of seeds P of the context (all blocks), or -1 for NULL. */

@@ -38,6 +38,7 @@ struct bto_ctx {
     int layout = bto::LAYOUT_F3;
     int nt = 128, ppt = 2, ctas_per_sm = 0, grid = 0;
     bool cap = false;         // cap registers at 80 (768 threads per SM)
+    bool shape_set = false;   // the launch shape is the caller's or the autotuner's
     size_t dyn_smem = 0;
     std::vector<BlockDev> blocks_h;
     BlockDev *blocks = nullptr;
@@ -252,7 +253,20 @@ bto::PartList part_list(const bto_ctx *c, int64_t first = 0) {
 //   from 0.75M   256 x 2, 80 registers (2.1M seeds, 20 cycles: 837 us against
 //       873; stride 2, 25 cycles, 1.49 ms against 1.52)
 //   between   128 x 2 (0.5M: 182 us against 190 at 128 x 1, 201 at 256 x 2)
+// With ingest every launch holds one block, so the largest block decides, and
+// gathering 16-byte nodes in cache moves the lines (us a cycle): 96 blocks of
+// 32,768 seeds 658 at 128 x 1, 815 at 128 x 2, 1035 at 256 x 4; 32 of 110,592
+// 335, 329, 407; 24 of 262,144 375, 344, 370; 8 of 884,736 330, 249, 246; one
+// of 4.1M 175, 121, 117.
 void default_shape(bto_ctx *c) {
+    if (c->ingest) {
+        int64_t most = 0;
+        for (const BlockDev &B : c->blocks_h) most = std::max(most, B.nseeds);
+        c->cap = most >= 750000;
+        c->nt = c->cap ? 256 : 128;
+        c->ppt = c->cap ? 4 : (most > 65536 ? 2 : 1);
+        return;
+    }
     const int64_t units = c->slots / bto::kUnit, resident = (int64_t)c->sm_count * 20;
     c->nt = 128;
     c->ppt = units <= 3 * resident ? 1 : 2;
@@ -727,7 +741,26 @@ bto_status bto_set_ingest(bto_ctx *ctx, int32_t enable) {
             BTO_CUDA(cudaEventCreateWithFlags(&ctx->adv_done[k], cudaEventDisableTiming));
         }
     }
+    const bool was = ctx->ingest;
+    const int o[3] = {ctx->nt, ctx->ppt, ctx->cap ? 1 : 0};
     ctx->ingest = enable != 0;
+    if (!ctx->shape_set && ctx->ingest != was) {
+        default_shape(ctx);
+        bto_status st = configure_launch(ctx);
+        if (st == BTO_OK && o[1] != ctx->ppt) {
+            // group counts depend on the group size: seed the interval afresh
+            st = cuda_status(cudaDeviceSynchronize());
+            if (st == BTO_OK) st = seed(ctx, 0);
+            if (st == BTO_OK) st = cuda_status(cudaDeviceSynchronize());
+        }
+        if (st != BTO_OK) {
+            (void)cudaGetLastError();
+            ctx->ingest = was;
+            ctx->nt = o[0]; ctx->ppt = o[1]; ctx->cap = o[2] != 0;
+            configure_launch(ctx);
+            return st;
+        }
+    }
     drop_graph(ctx);
     return BTO_OK;
 }
@@ -869,6 +902,7 @@ bto_status bto_set_launch(bto_ctx *ctx, int32_t threads_per_cta, int32_t particl
         return st;
     }
     drop_graph(ctx);
+    ctx->shape_set = true;
     if (o[1] != ctx->ppt) {
         // group counts depend on the group size: seed the interval afresh
         BTO_CUDA(cudaDeviceSynchronize());
@@ -987,6 +1021,7 @@ bto_status bto_autotune(bto_ctx *ctx, const void *const *d_field_table, int32_t 
         ctx->ppt = shapes[best_k][1];
         ctx->ctas_per_sm = 0;
         ctx->cap = shapes[best_k][2] != 0;
+        ctx->shape_set = true;
     } else {
         ctx->nt = keep[0]; ctx->ppt = keep[1]; ctx->ctas_per_sm = keep[2]; ctx->cap = keep[3] != 0;
     }
