@@ -505,7 +505,8 @@ BTO_API bto_status bto_set_device_allocator(bto_alloc_fn alloc, bto_free_fn free
 /* ---- Bounds-checked builds (no counterpart in the paper) ----------------
  *
  * Compiled with BTO_CHECK_BOUNDS defined (build.build(check_bounds=True)),
- * the kernels test every field-node index of a global gather, every group
+ * the kernels test every field-node index of a global gather, of a row
+ * touched ahead and of the tape's gradient sums, every group
  * count and particle id of the particle list, every destination tile of the
  * tiled path and every lattice index of the post hoc kernels before using
  * it. A failed test skips the access (a node or lattice index is replaced by

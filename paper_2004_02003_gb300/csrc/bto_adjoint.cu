@@ -133,7 +133,7 @@ __device__ __forceinline__ void sample_jac(JCell &C, const float *__restrict__ f
     cell_coord_any(z, g.cmz, st.iz, st.fz);
     const uint32_t node = (uint32_t)st.ix + g.nnx * (uint32_t)st.iy + g.nnxy * (uint32_t)st.iz;
     if (node != C.node) {
-        load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, st.ix, st.iy, st.iz, C.v);
+        load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, g.nodes, st.ix, st.iy, st.iz, C.v);
         C.node = node;
     }
     const float (&c)[8][3] = C.v;
@@ -304,6 +304,7 @@ __device__ __forceinline__ void add_cell(float *__restrict__ gF, const Geo &g, u
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
+        if (!BTO_IN_BOUNDS((uint64_t)nd + 1 < g.nodes, nullptr)) continue;
         float *p = gF + 3ull * nd;
         const float *a = v[2 * q], *b = v[2 * q + 1];
         const bool odd = (reinterpret_cast<uintptr_t>(p) & 4u) != 0;
@@ -328,7 +329,7 @@ __device__ __forceinline__ void locate(JCell &C, const float *__restrict__ f, co
     cell_coord_any(x.z, g.cmz, iz, fz);
     const uint32_t node = (uint32_t)ix + g.nnx * (uint32_t)iy + g.nnxy * (uint32_t)iz;
     if (node != C.node) {
-        load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, ix, iy, iz, C.v);
+        load_cell<bto::LAYOUT_F3>(f, g.nnx, g.nnxy, g.nodes, ix, iy, iz, C.v);
         C.node = node;
     }
 }
@@ -741,6 +742,10 @@ bto_status tangents(const bto_tape *t, cudaStream_t s) {
 }
 
 }  // namespace
+
+namespace bto {
+BTO_BOUNDS_ACCESSOR(bounds_failures_adjoint)
+}
 
 extern "C" {
 

@@ -1182,9 +1182,10 @@ int32_t bto_check_bounds_build(void) {
 
 bto_status bto_bounds_failures(uint64_t *count, int32_t reset) {
     if (!count) return BTO_ERR_INVALID_ARG;
-    const unsigned long long parts[4] = {bto::bounds_failures_kernels(reset != 0), bto::bounds_failures_tiled(reset != 0),
+    const unsigned long long parts[5] = {bto::bounds_failures_kernels(reset != 0), bto::bounds_failures_tiled(reset != 0),
                                          bto::bounds_failures_posthoc(reset != 0),
-                                         bto::bounds_failures_delaunay(reset != 0)};
+                                         bto::bounds_failures_delaunay(reset != 0),
+                                         bto::bounds_failures_adjoint(reset != 0)};
     uint64_t total = 0;
     for (const unsigned long long v : parts) {
         if (v == ~0ull) {

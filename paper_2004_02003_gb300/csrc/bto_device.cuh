@@ -23,8 +23,12 @@ __device__ __forceinline__ float lerp1(float a, float b, float t) { return fmaf(
 // the adjoint's sampler, which also differentiates the weights.
 template <int LAYOUT>
 __device__ __forceinline__ void load_cell(const void *__restrict__ field, uint32_t nnx,
-                                          uint32_t nnxy, int ix, int iy, int iz,
+                                          uint32_t nnxy, uint32_t nodes, int ix, int iy, int iz,
                                           float (&v)[8][3]) {
+    // the cell's last corner must be a node of the block
+    if (!BTO_IN_BOUNDS((uint64_t)(uint32_t)ix + 1 + (uint64_t)nnx * (uint32_t)(iy + 1) +
+                           (uint64_t)nnxy * (uint32_t)(iz + 1) < nodes, nullptr))
+        ix = iy = iz = 0;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -317,10 +321,12 @@ __device__ __forceinline__ uint32_t near_cell(const Geo &g, float x, float y, fl
 // shared memory that nobody reads. A plain load would hold a register and a
 // scoreboard; prefetch.global.L1 and .L2 measured half the gain and none.
 template <int LAYOUT>
-__device__ __forceinline__ void touch_row(const void *__restrict__ field, const Geo &g, uint32_t node, uint32_t word) {
+__device__ __forceinline__ void touch_row(const void *__restrict__ field, const Geo &g, uint32_t node, uint32_t word,
+                                          int32_t *err) {
     constexpr uint32_t kNode = LAYOUT == LAYOUT_F4 ? 16 : 12;
     const int q = threadIdx.x & 3;
     const uint32_t nd = node + ((q & 1) ? g.nnx : 0u) + ((q & 2) ? g.nnxy : 0u);
+    if (!BTO_IN_BOUNDS((uint64_t)nd + 1 < g.nodes, err)) return;
     const char *p = reinterpret_cast<const char *>(field) + (uint64_t)kNode * nd;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(word), "l"(p) : "memory");
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(word), "l"(p + 2 * kNode - 4) : "memory");
@@ -354,12 +360,12 @@ __device__ __forceinline__ int rk4_step_quad(float3 &x, const void *__restrict__
         const float3 v = sample_quad<LAYOUT>(C, field, g, on, px, py, pz, err);
         if (k == 0 && on) {
             const uint32_t n1 = near_cell(g, fmaf(s.x, v.x, x.x), fmaf(s.y, v.y, x.y), fmaf(s.z, v.z, x.z));
-            if (n1 != C.node) touch_row<LAYOUT>(field, g, n1, ahead.word);
+            if (n1 != C.node) touch_row<LAYOUT>(field, g, n1, ahead.word, err);
             if (ahead.next) {
-                touch_row<LAYOUT>(ahead.next, g, n1, ahead.word);
+                touch_row<LAYOUT>(ahead.next, g, n1, ahead.word, err);
                 const uint32_t n2 = near_cell(g, fmaf(1.5f * s.x, v.x, x.x), fmaf(1.5f * s.y, v.y, x.y),
                                               fmaf(1.5f * s.z, v.z, x.z));
-                if (n2 != n1) touch_row<LAYOUT>(ahead.next, g, n2, ahead.word);
+                if (n2 != n1) touch_row<LAYOUT>(ahead.next, g, n2, ahead.word, err);
             }
         }
         if (k == 0) acc = v;

@@ -81,6 +81,7 @@ unsigned long long bounds_failures_kernels(bool reset);
 unsigned long long bounds_failures_tiled(bool reset);
 unsigned long long bounds_failures_posthoc(bool reset);
 unsigned long long bounds_failures_delaunay(bool reset);
+unsigned long long bounds_failures_adjoint(bool reset);
 
 // One block of the uniform grid, as the kernels see it. Positions inside the
 // library are block-local CELL coordinates xi = (x - origin) / h, so node i

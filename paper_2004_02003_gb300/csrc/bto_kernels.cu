@@ -191,8 +191,9 @@ __global__ void __launch_bounds__(kRegionAlign, kIntervalCtas) interval_kernel(c
     const int per = group / kUnit;                           // units of a group
     const int first = warp / per * per;                      // first unit of this warp's group, in the CTA
     const int64_t grp = (s0 + first * kUnit) / group;
-    int cnt = a.p.gcnt[grp] - (warp - first) * kUnit;        // live particles from this unit on
-    if (!BTO_IN_BOUNDS(cnt <= group, a.err)) cnt = 0;
+    int cnt = a.p.gcnt[grp];
+    if (!BTO_IN_BOUNDS(cnt >= 0 && cnt <= group, a.err)) cnt = 0;
+    cnt -= (warp - first) * kUnit;                           // live particles from this unit on
     const int b = a.gblock[unit];
     const BlockDev &B = a.blocks[b];
     const Geo g = load_geo(B);
