@@ -141,7 +141,7 @@ def _addr(buf) -> int:
         return None
     if isinstance(buf, int):
         return buf
-    return buf.data_ptr()
+    return int(buf.data_ptr())
 
 
 _torch = None
