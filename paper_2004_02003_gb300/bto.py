@@ -144,22 +144,38 @@ def _addr(buf) -> int:
     return int(buf.data_ptr())
 
 
-_torch = None
+_current = None
+
+
+def _bind_current():
+    """A function that gives the address of torch's current stream on the
+    current device. By its raw handle where torch has the calls for it (they
+    are not public): building a Stream object took 1.5 of the 6.6 us of a
+    per-cycle call, which is what bounds the cycles of a small block."""
+    import torch
+
+    def by_object():
+        return torch.cuda.current_stream().cuda_stream
+
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return by_object
+    ready = torch.cuda.is_initialized
+
+    def by_handle():
+        return raw(device()) if ready() else by_object()
+
+    return by_handle
 
 
 def _stream(stream):
-    """The stream's address. Without one, torch's current stream on the
-    current device, asked for by its raw handle: building a Stream object for
-    it took 1.5 of the 6.6 us of a per-cycle call, which is what bounds the
-    cycles of a small block."""
+    """The stream's address; torch's current stream without one."""
     if stream is None:
-        global _torch
-        if _torch is None:
-            import torch
-            _torch = torch
-        if not _torch.cuda.is_initialized():
-            return _torch.cuda.current_stream().cuda_stream
-        return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
+        global _current
+        if _current is None:
+            _current = _bind_current()
+        return _current()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
