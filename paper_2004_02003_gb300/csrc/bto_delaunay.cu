@@ -1217,51 +1217,36 @@ constexpr int kCopyTile = 4 * kFillThreads;   // entries of a CTA of the copy
 // Tiles for each CTA in flight from which on those with missing entries are
 // listed: below, the few waves of CTAs that find nothing cost no more than the
 // list's memset (33 x 31 x 29, none missing: 16 us either way). 64^3, none
-// missing: 14 us, 26 with a CTA to copy and look through each tile; 256^3: 89
+// missing: 17 us, 26 with a CTA to copy and look through each tile; 256^3: 93
 // and 1,310.
 constexpr int kListTiles = 4;
 constexpr int kTileN = kTileX * kTileY * kTileZ;
 
 // How the solver's tiles are listed: groups of w tiles along x by v along z,
-// group (bx / w, by, bz / v) number bx / w + gx (by + ty (bz / v)).
-// w == 0: no list.
+// group (bx / w, by, bz / v) number bx / w + gx (by + ty (bz / v)). w == 0: no
+// list. The lists stand in the out entries of the plane z = 0, which are
+// written last (by the boundary kernel): words 0 to 2 are the groups with
+// missing interior entries, those with kDense or more, and the tiles the
+// solver has taken; then the groups' counts of missing interior entries, two
+// to a word, and the two lists, n words each.
 struct Groups {
     int tx, ty, tz;   // tiles per axis
     int w, v;
     int gx;           // groups along x
+    int n;            // groups
 };
+// Missing entries from which on a group counts as dense, of 128 and more: over
+// 24 lattices of 24 to 112 points an axis with losses at block faces, each with
+// two inputs, the fill takes 0.963 of the time with a CTA to each tile in
+// lattice order (0.985 at 3, 0.970 at 5, 0.972 at 12, 0.997 at 24, 1.017
+// without the order); 128^3 4.86 ms against 5.12.
+constexpr int kDense = 8;
+__host__ __device__ inline int64_t list_words(int64_t n) { return 3 + (n + 1) / 2 + 2 * n; }
 
-// Whether no interior entry of its group before (x, y, z), in lattice order,
-// is missing. Missing entries come in slabs: its neighbours first, then its
-// own row backward.
-__device__ __forceinline__ bool first_of_group(int3 S, const uint8_t *__restrict__ valid, const Groups &G, int x, int y,
-                                               int z) {
-    const int ex = kTileX * G.w, ez = kTileZ * G.v;
-    const int x0 = max(x / ex * ex, 1), x1 = min(x / ex * ex + ex, S.x - 1);   // x1 and y1: one past
-    const int y0 = max(y / kTileY * kTileY, 1), y1 = min(y / kTileY * kTileY + kTileY, S.y - 1);
-    const int z0 = max(z / ez * ez, 1);
-    const uint8_t *row = valid + lattice_rank(S, 0, y, z);
-    if ((y > y0 && !row[x - S.x]) || (z > z0 && !row[x - (int64_t)S.x * S.y])) return false;
-    for (int k = x - 1; k >= x0; --k)
-        if (!row[k]) return false;
-    for (int zz = z; zz >= z0; --zz)
-        for (int yy = (zz == z ? y : y1) - 1; yy >= y0; --yy) {
-            row = valid + lattice_rank(S, 0, yy, zz);
-            bool all = true;
-#pragma unroll 8
-            for (int k = x0; k < x1; ++k) all = all && row[k] != 0;
-            if (!all) return false;
-        }
-    return true;
-}
-
-// Copies the valid entries (status 1) and lists the groups that hold missing
-// interior entries, each by the first of them. The list stands in the out
-// entries of the plane z = 0, which are written last (by the boundary
-// kernel): word 0 counts the groups, word 1 the tiles the solver has taken,
-// the groups follow. On a lattice one point thick, which has no tetrahedra,
-// the missing entries are finished here. Bound by HBM: 16-byte accesses where
-// the pointers allow it.
+// Copies the valid entries (status 1), counts the groups' missing interior
+// entries and lists the groups by their first and their kDense-th. On a
+// lattice one point thick, which has no tetrahedra, the missing entries are
+// finished here. Bound by HBM: 16-byte accesses where the pointers allow it.
 template <bool VEC>
 __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const Groups G, bool flat,
                                                                  const float *__restrict__ ends,
@@ -1317,9 +1302,12 @@ __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const G
         const unsigned p32 = (unsigned)p, r = p32 / (unsigned)S.x;   // below 2^31
         const int x = (int)(p32 - r * (unsigned)S.x), y = (int)(r % (unsigned)S.y), z = (int)(r / (unsigned)S.y);
         if (x < 1 || x >= S.x - 1 || y < 1 || y >= S.y - 1 || z < 1 || z >= S.z - 1) continue;
-        if (!first_of_group(S, valid, G, x, y, z)) continue;
-        unsigned *list = reinterpret_cast<unsigned *>(out);
-        list[2 + atomicAdd(list, 1u)] = (unsigned)(x / (kTileX * G.w) + G.gx * (y / kTileY + G.ty * (z / (kTileZ * G.v))));
+        const unsigned g = (unsigned)(x / (kTileX * G.w) + G.gx * (y / kTileY + G.ty * (z / (kTileZ * G.v))));
+        unsigned *head = reinterpret_cast<unsigned *>(out), *counts = head + 3, *list = counts + (G.n + 1) / 2;
+        const int sh = (g & 1) * 16;
+        const unsigned before = atomicAdd(counts + g / 2, 1u << sh) >> sh & 0xffffu;
+        if (before == 0) list[atomicAdd(head, 1u)] = g;
+        if (before == kDense - 1) list[G.n + atomicAdd(head + 1, 1u)] = g;
     }
 }
 
@@ -1330,8 +1318,10 @@ __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const G
 // tile is what its four warps work through alone (8 x 4 x 2: 6.5 ms where this
 // took 5.8, 16 x 4 x 4 a millisecond more again), and no smaller, since its
 // entries share the words (8 x 2 x 1: 5.36 ms where this took 5.14). LISTED:
-// the CTAs in flight take the tiles of the listed groups from a counter; else
-// every tile has a CTA, and the hardware hands them out.
+// the CTAs in flight take the tiles of the listed groups from a counter, the
+// dense groups' first, since a tile full of missing entries that starts late
+// is what the call then waits for; else every tile has a CTA, and the
+// hardware hands them out.
 // Bound by instructions: about 1,400 a pivot, a straight run of code far
 // longer than the instruction caches hold (most stalls are instruction
 // fetch), 16 pivots an entry. A 128^3 lattice with 137,210 missing entries
@@ -1354,8 +1344,10 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    unsigned *listed = reinterpret_cast<unsigned *>(out);
-    const unsigned sub = (unsigned)(G.w * G.v), total = LISTED ? __ldcg(listed) * sub : 0u;
+    unsigned *head = reinterpret_cast<unsigned *>(out);
+    const unsigned *counts = head + 3, *list_of = counts + (G.n + 1) / 2;
+    const unsigned sub = (unsigned)(G.w * G.v), dense = LISTED ? __ldcg(head + 1) * sub : 0u,
+                   total = LISTED ? dense + __ldcg(head) * sub : 0u;
 #pragma unroll 1
     for (;;) {
         if (warp == 0) {
@@ -1363,16 +1355,18 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, 
             if (LISTED) {
                 unsigned job = 0, g = 0;
                 if (lane == 0) {
-                    job = atomicAdd(listed + 1, 1u);
-                    if (job < total) g = __ldcg(listed + 2 + job / sub);
+                    job = atomicAdd(head + 2, 1u);
+                    if (job < dense) g = __ldcg(list_of + G.n + job / sub);
+                    else if (job < total) g = __ldcg(list_of + (job - dense) / sub);
                 }
                 job = __shfl_sync(kAll, job, 0);
                 g = __shfl_sync(kAll, g, 0);
-                const int in = (int)(job % sub);
+                const int in = (int)((job < dense ? job : job - dense) % sub);
                 bx = (int)(g % (unsigned)G.gx) * G.w + in % G.w;
                 by = (int)(g / (unsigned)G.gx % (unsigned)G.ty);
                 bz = (int)(g / (unsigned)G.gx / (unsigned)G.ty) * G.v + in / G.w;
                 if (job >= total) bx = -1;   // none left
+                else if (job >= dense && (__ldcg(counts + g / 2) >> (g & 1) * 16 & 0xffffu) >= kDense) bx = G.tx;   // taken
             } else {
                 bx = (int)(blockIdx.x % G.tx);
                 by = (int)(blockIdx.x / G.tx % G.ty);
@@ -1538,18 +1532,21 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, int
 
 BTO_BOUNDS_ACCESSOR(bounds_failures_delaunay)
 
-// The solver's groups, and whether their list fits the plane z = 0 of out.
-static Groups groups_of(const int32_t S[3], bool listed) {
+// The solver's groups: as few tiles along z to a group as let the lists fit
+// the plane z = 0 of out.
+static Groups groups_of(const int32_t S[3]) {
     Groups G{};
     G.tx = (S[0] + kTileX - 1) / kTileX;
     G.ty = (S[1] + kTileY - 1) / kTileY;
     G.tz = (S[2] + kTileZ - 1) / kTileZ;
-    if (!listed) return G;
     G.w = G.tx < 4 ? G.tx : 4;
     G.gx = (G.tx + G.w - 1) / G.w;
-    const int64_t room = (3 * (int64_t)S[0] * S[1] - 2) / ((int64_t)G.gx * G.ty);   // groups along z: 1 or more
-    const int64_t gz = room < G.tz ? room : G.tz;
+    const int64_t per = (int64_t)G.gx * G.ty, words = 3 * (int64_t)S[0] * S[1];
+    int64_t gz = (words - 4) * 2 / 5 / per;
+    if (gz > G.tz) gz = G.tz;
+    if (gz < 1) gz = 1;
     G.v = (int)((G.tz + gz - 1) / gz);
+    G.n = (int)(per * ((G.tz + G.v - 1) / G.v));
     return G;
 }
 
@@ -1577,11 +1574,15 @@ cudaError_t launch_fill_delaunay(const int32_t S[3], const float *ends, const ui
     const int64_t tiles = (int64_t)((S[0] + kTileX - 1) / kTileX) * ((S[1] + kTileY - 1) / kTileY) * ((S[2] + kTileZ - 1) / kTileZ);
     const int64_t resident = 4ll * sm_count;
     const bool apart = out + 3 * P <= ends || ends + 3 * P <= out;   // the list would spoil ends
-    const bool listed = inner && apart && tiles > kListTiles * resident;
-    const Groups G = groups_of(S, listed);
+    Groups G = groups_of(S);
+    // a group's count has 16 bits
+    const bool listed = inner && apart && tiles > kListTiles * resident && list_words(G.n) <= 3 * (int64_t)S[0] * S[1] &&
+                        (int64_t)kTileN * G.w * G.v < 65536;
     if (listed) {
-        const cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(uint32_t), s);
+        const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(uint32_t) * (3 + (G.n + 1) / 2), s);
         if (e != cudaSuccess) return e;
+    } else {
+        G.w = 0;
     }
     const unsigned copies = (unsigned)((P + kCopyTile - 1) / kCopyTile);
     const bool vec = !((reinterpret_cast<uintptr_t>(ends) | reinterpret_cast<uintptr_t>(out)) & 15u) &&
