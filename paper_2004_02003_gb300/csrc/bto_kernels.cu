@@ -171,18 +171,24 @@ __global__ void __launch_bounds__(NT, MINB) advect_kernel(const AdvectArgs a) {
 // per-cycle launch would have left them. A CTA is four units: a region is a
 // multiple of 128 slots, so a CTA lies in one block and holds whole groups.
 // Against a graph of one launch per cycle this drops the launches, their
-// tails and the list's 24 bytes per particle and cycle: one 64^3 block with
-// 10,648 seeds over 100 cycles 648 -> 206 us (bound by the latency of its
-// dependent samples, 2 warps per SM), 96 blocks of 16 to 96 cells with 7.5M
-// seeds over 32 cycles 5.15 -> 3.95 ms (bound by the L1 load path).
+// tails and the list's 24 bytes per particle and cycle: 96 blocks of 16 to 96
+// cells with 7.5M seeds over 32 cycles 5.15 -> 3.76 ms (bound by the L1 load
+// path). Short lists, which this leaves waiting for dependent samples, take
+// interval_quad_kernel.
 // ---------------------------------------------------------------------------
-// Eight CTAs of 128 per SM (64 registers, 32 bytes spilled): 3.76 ms on the
-// 96 blocks against 3.92 at the compiler's own 72 registers, 4.80 at nine.
-constexpr int kIntervalCtas = 8;
+// CTAs of 128 per SM. F3: eight (64 registers, 20 bytes spilled); 3.76 ms on
+// the 96 blocks against 3.92 at the compiler's own 72 registers, 4.80 at nine,
+// and 885 us against 891 at seven on 200^3 cells seeded 1:1 over 8 cycles. F4:
+// seven (72 registers, 28 bytes spilled; 64 spill 56): 3.45 ms against 3.67 at eight
+// and 3.60 at six on 96 such blocks, 973 us against 1000 and 1029 on the 200^3,
+// 194 against 208 and 215 on 20 blocks of 24 to 40 cells over 40 cycles.
+template <int LAYOUT>
+constexpr int kIntervalCtas = LAYOUT == LAYOUT_F4 ? 7 : 8;
 
 template <int LAYOUT>
-__global__ void __launch_bounds__(kRegionAlign, kIntervalCtas) interval_kernel(const AdvectArgs a, const int32_t cycles,
-                                                                const int group) {
+__global__ void __launch_bounds__(kRegionAlign, kIntervalCtas<LAYOUT>) interval_kernel(const AdvectArgs a,
+                                                                                        const int32_t cycles,
+                                                                                        const int group) {
     static_assert(kRegionAlign == 4 * kUnit, "a CTA is four units");
     __shared__ int kept[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -248,7 +254,10 @@ __global__ void __launch_bounds__(kRegionAlign, kIntervalCtas) interval_kernel(c
     if (warp == first && lane == 0) a.p.gcnt[grp] = total;
 }
 
-// The same by four lanes per particle (rk4_step_quad): a CTA is one group.
+// The same by four lanes per particle (rk4_step_quad): a CTA is one group. One
+// 64^3 block with 10,648 seeds over 100 cycles: 648 us in a graph of one launch
+// per cycle, 212 by interval_kernel (2 warps per SM), 121 so; bound by the
+// latency of the dependent samples.
 template <int LAYOUT>
 __global__ void __launch_bounds__(4 * kRegionAlign) interval_quad_kernel(const AdvectArgs a, const int32_t cycles,
                                                                          const int group) {
