@@ -54,7 +54,7 @@ struct bto_ctx {
     cudaGraphExec_t gexec = nullptr;
     const void *const *gtable = nullptr;
     float gdt = 0.f;
-    int gshape[5] = {0, 0, 0, 0, 0};
+    int glayout = -1;
     int gtiling = -1;
     cudaStream_t capture_stream = nullptr;
     // H1 ingest (F3 fields repacked to F4 per block, two buffers in flight)
@@ -810,9 +810,7 @@ bto_status bto_launch_interval_graph(bto_ctx *ctx, const void *const *d_field_ta
         return BTO_OK;
     }
     const bool same = ctx->gexec && ctx->gtable == d_field_table && ctx->gdt == dt &&
-                      ctx->gshape[0] == ctx->layout && ctx->gshape[1] == ctx->nt &&
-                      ctx->gshape[2] == ctx->ppt && ctx->gshape[3] == ctx->grid &&
-                      ctx->gshape[4] == (ctx->cap ? 1 : 0) && ctx->gtiling == ctx->tiling_gen;
+                      ctx->glayout == ctx->layout && ctx->gtiling == ctx->tiling_gen;
     if (!same) {
         drop_graph(ctx);
         if (!ctx->capture_stream)
@@ -839,11 +837,7 @@ bto_status bto_launch_interval_graph(bto_ctx *ctx, const void *const *d_field_ta
         }
         ctx->gtable = d_field_table;
         ctx->gdt = dt;
-        ctx->gshape[0] = ctx->layout;
-        ctx->gshape[1] = ctx->nt;
-        ctx->gshape[2] = ctx->ppt;
-        ctx->gshape[3] = ctx->grid;
-        ctx->gshape[4] = ctx->cap ? 1 : 0;
+        ctx->glayout = ctx->layout;
         ctx->gtiling = ctx->tiling_gen;
     }
     BTO_CUDA(cudaGraphLaunch(ctx->gexec, (cudaStream_t)stream));
