@@ -665,7 +665,7 @@ def extras(args, ctx, fields, gfields, table, out, exit_ref, psteps, dt, dev, st
 
 def adjoint_leg(args, dev, stream):
     """Adjoint workload (64^3 ABC block on [0, 2 pi]^3, 32^3 seeds, 200 cycles,
-    dt 0.01, checkpoints every 16): the plain interval against the tape's
+    dt 0.01): the plain interval against the tape's
     forward and forward + backward (seed and node-velocity gradients of
     sum over valid particles of |end - seed|^2), same GPU, same fields."""
     import torch
@@ -719,7 +719,7 @@ def adjoint_leg(args, dev, stream):
     psteps = count_particle_steps(ex, L)
     tape.close()
     ctx.close()
-    return {"workload": "64^3 ABC on [0,2pi]^3, 32,768 seeds (stride 2), 200 cycles, dt 0.01, checkpoints every 16",
+    return {"workload": "64^3 ABC on [0,2pi]^3, 32,768 seeds (stride 2), 200 cycles, dt 0.01",
             "plain_ms": t_plain, "tape_forward_ms": t_fwd, "forward_backward_ms": t_fb,
             "forward_backward_vs_plain": t_fb / t_plain,
             "plain_particle_steps_per_s": psteps / (t_plain / 1e3),

@@ -5,12 +5,13 @@
 F3 node field per cycle) with one RK4 step per cycle and closed-box
 termination (Sec. 3.1), and returns the end positions (the basis flows,
 Sec. 2.3), the valid flags and the exit cycles. Its backward pass runs the
-checkpointed discrete adjoint kernels of libbto and returns the gradients
+discrete adjoint kernels of libbto and returns the gradients
 with respect to the seeds and to every cycle's node velocities. Only
 argument marshalling happens here; all arithmetic runs in libbto.
 
-``ftle(tape, seeds, fields, dt)`` returns the flow-map Jacobian and the finite-time Lyapunov exponent of every particle that
-stays in its block for the interval.
+``ftle(tape, seeds, fields, dt)`` returns the flow-map Jacobian and the
+finite-time Lyapunov exponent of every particle that stays in its block for the
+interval.
 """
 from __future__ import annotations
 

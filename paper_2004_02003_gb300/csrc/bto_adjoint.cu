@@ -728,8 +728,10 @@ dim3 seg_grid(const bto_tape *t) {
 
 // Cycles per segment, from the interval alone (so that the rounding of the
 // results does not depend on checkpoint_every): 1.2 sqrt(L), at least 4. The
-// tape then holds 52 nseg = 43 sqrt(L) bytes a particle, less than a serial
-// sweep's checkpoints and segment positions take at any spacing.
+// tape then holds 52 nseg = 43 sqrt(L) bytes a particle. A serial sweep with a
+// checkpoint every K cycles, three rows of K positions to recompute a segment
+// for the Jacobian, and three adjoints took 16 (L / K + 3 K + 4), which is 55
+// sqrt(L) + 64 at the best K.
 int32_t segment_cycles(int32_t L) {
     return std::max<int32_t>(4, (int32_t)std::ceil(1.2 * std::sqrt((double)L)));
 }

@@ -243,16 +243,22 @@ bto::PartList part_list(const bto_ctx *c, int64_t first = 0) {
 }
 
 // The launch shape of a new context (bto_set_launch and bto_autotune change
-// it), by the particles it holds; 152 SMs of 20 resident warps are meant:
+// it), by the particles it holds; 152 SMs of 20 resident warps are meant. Over
+// 0.11M to 16.8M seeds in 1 to 96 blocks, F3 and F4, it is at most 1.5% behind
+// 128 x 2 (8 blocks of 160^3 at stride 2: 127.8 us a cycle against 126.0) and
+// mostly 3 to 15% ahead:
 //   up to three rounds of one 32-slot unit per warp   128 threads x 1: a warp's
 //       units run one after another, and two to a warp leave the last round
 //       half empty (64^3 cells, 262,144 seeds: 183 us against 209 of 20 cycles)
 //   from 3M   256 x 4, 80 registers: four units' records are in flight at
 //       once (16.8M seeds, 10 cycles: 2.71 ms against 3.17 at 128 x 2; F4
-//       fields, 8 cycles, 2.35 against 3.07; 2.1M: 885 us against 873)
+//       fields, 8 cycles, 2.35 against 3.07; a cycle of 4.1M 83.9 us against
+//       84.4 at 256 x 2, of 3.0M 65.0 against 63.7)
 //   from 0.75M   256 x 2, 80 registers (2.1M seeds, 20 cycles: 837 us against
-//       873; stride 2, 25 cycles, 1.49 ms against 1.52)
-//   between   128 x 2 (0.5M: 182 us against 190 at 128 x 1, 201 at 256 x 2)
+//       873; stride 2, 25 cycles, 1.49 ms against 1.52; a cycle of 0.88M 22.7
+//       us against 23.8)
+//   between   128 x 2 (0.5M: 182 us against 190 at 128 x 1, 201 at 256 x 2; a
+//       cycle of 0.68M 19.9 us, 19.2 at either)
 // With ingest every launch holds one block, so the largest block decides, and
 // gathering 16-byte nodes in cache moves the lines (us a cycle): 96 blocks of
 // 32,768 seeds 658 at 128 x 1, 815 at 128 x 2, 1035 at 256 x 4; 32 of 110,592

@@ -164,12 +164,8 @@ __device__ __forceinline__ bool positive_range(int64_t a, int64_t b, int64_t lo,
     return t0 <= t1;
 }
 
-// Outcome of one walk in a window of radius R around the lattice point c:
-// 1 and the tetrahedron with q's barycentric coordinates, or 0 (no result
-// in this window: q outside the hull of its valid points, circumsphere
-// larger than the window, or the pivot limit).
-// Circumsphere of T (centre and squared radius, FP64), for the filter that
-// spares most points the exact predicate.
+// Circumsphere of T (centre and squared radius, FP64), for the test whether it
+// fits the window where FP32 leaves that open.
 __device__ __noinline__ void circumsphere(const LPt (&T)[4], double (&ctr)[3], double &r2) {
     double A[3][3], b[3];
     const LPt &a = T[0];
@@ -563,7 +559,10 @@ __device__ __noinline__ bool across_facet(int3 S, const uint8_t *__restrict__ va
 // from the point nearest to the centre outward, in FP32 too (rounding is
 // monotone), so a lane walks outward from there on both sides and stops as
 // soon as the depth is below its best. Only points that would become the
-// lane's best get the exact predicate.
+// lane's best get the exact predicate. Returns 1 and the tetrahedron with q's
+// barycentric coordinates, or 0: no result in this window (q outside the hull
+// of its valid points, circumsphere larger than the window, or the pivot
+// limit).
 __device__ __forceinline__ int walk(int3 S, const uint8_t *__restrict__ valid, const uint32_t *win, int lx, int cx, int cy,
                                  int cz, int R, bool &settled, LPt (&T)[4], double (&lam)[4]) {
     const int lane = threadIdx.x & 31;
@@ -819,7 +818,7 @@ __device__ __forceinline__ int perturbed_sign2(const LPt2 (&t)[3], const LPt2 &e
     return sign;
 }
 
-// Circumcircle of T (centre and squared radius, FP64), for the filter.
+// Circumcircle of T (centre and squared radius, FP64), as circumsphere.
 __device__ __noinline__ void circumcircle(const LPt2 (&T)[3], double (&ctr)[2], double &r2) {
     const double bx = (double)(T[1].u - T[0].u), by = (double)(T[1].v - T[0].v);
     const double cx = (double)(T[2].u - T[0].u), cy = (double)(T[2].v - T[0].v);
@@ -831,8 +830,8 @@ __device__ __noinline__ void circumcircle(const LPt2 (&T)[3], double (&ctr)[2], 
     r2 = ux * ux + uy * uy;
 }
 
-// The circumcircle of T for the face walk's filter, as circumsphere_f:
-// exact 64-bit Cramer numerators, FP32 quotients.
+// The circumcircle of T for the face walk's filter, as in sphere_of: exact
+// 64-bit Cramer numerators, FP32 quotients.
 __device__ __forceinline__ void circumcircle_f(const LPt2 (&T)[3], float (&c)[2], float &r2) {
     const int64_t bx = T[1].u - T[0].u, by = T[1].v - T[0].v, cx = T[2].u - T[0].u, cy = T[2].v - T[0].v;   // below 2^12
     const int64_t b2 = bx * bx + by * by, c2 = cx * cx + cy * cy;
@@ -1132,7 +1131,7 @@ __device__ __forceinline__ int walk2(int3 S, const uint8_t *__restrict__ valid, 
         const LPt2 e = {(int32_t)(f.a == 0 ? bc[0] : bc[1]) - f.ca, (int32_t)(f.b == 1 ? bc[1] : bc[2]) - f.cb, (uint32_t)best};
         int leave = -1;
         int64_t bq = 0, be = 0;
-            uint32_t brank = 0;
+        uint32_t brank = 0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             LPt2 u[3] = {T[0], T[1], T[2]};

@@ -179,9 +179,9 @@ __global__ void __launch_bounds__(NT, MINB) advect_kernel(const AdvectArgs a) {
 // CTAs of 128 per SM. F3: eight (64 registers, 20 bytes spilled); 3.76 ms on
 // the 96 blocks against 3.92 at the compiler's own 72 registers, 4.80 at nine,
 // and 885 us against 891 at seven on 200^3 cells seeded 1:1 over 8 cycles. F4:
-// seven (72 registers, 28 bytes spilled; 64 spill 56): 3.45 ms against 3.67 at eight
-// and 3.60 at six on 96 such blocks, 973 us against 1000 and 1029 on the 200^3,
-// 194 against 208 and 215 on 20 blocks of 24 to 40 cells over 40 cycles.
+// seven (72 registers, 28 bytes spilled; 64 spill 56): 3.45 ms against 3.67 at
+// eight and 3.60 at six on 96 such blocks, 973 us against 1000 and 1029 on the
+// 200^3, 194 against 208 and 215 on 20 blocks of 24 to 40 cells over 40 cycles.
 template <int LAYOUT>
 constexpr int kIntervalCtas = LAYOUT == LAYOUT_F4 ? 7 : 8;
 
