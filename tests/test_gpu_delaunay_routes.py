@@ -90,3 +90,26 @@ def test_flat_lattice(S, shift):
     ok = valid != 0
     assert np.array_equal(out[ok], ends[ok]) and np.isnan(out[~ok]).all()
     assert np.array_equal(st, valid)
+
+
+# Captured into a CUDA graph, the fill's launches and the list's clearing replay
+# on whatever the buffers then hold.
+@pytest.mark.parametrize("S", [(67, 45, 53), (33, 31, 29), (40, 1, 25)])
+def test_fill_replays_from_a_captured_graph(S):
+    import torch
+    P = int(np.prod(S))
+    ends, valid = torch.zeros((P, 3), device="cuda"), torch.ones(P, dtype=torch.uint8, device="cuda")
+    out, st = torch.empty_like(ends), torch.empty_like(valid)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        bto.bto_fill_delaunay(S, ends, valid, out, st)
+    for holes in ("slabs", "none", "sparse"):
+        e, v = _lattice(S, holes, 5)
+        ends.copy_(torch.from_numpy(e))
+        valid.copy_(torch.from_numpy(v))
+        graph.replay()
+        want, st_want = torch.empty_like(ends), torch.empty_like(valid)
+        torch.cuda.synchronize()
+        bto.bto_fill_delaunay(S, ends, valid, want, st_want)
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int32), want.view(torch.int32)) and torch.equal(st, st_want)
