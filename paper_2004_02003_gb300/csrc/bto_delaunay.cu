@@ -1216,36 +1216,43 @@ constexpr int kCopyTile = 4 * kFillThreads;   // entries of a CTA of the copy
 // Tiles for each CTA in flight from which on those with missing entries are
 // listed: below, the few waves of CTAs that find nothing cost no more than the
 // list's memset (33 x 31 x 29, none missing: 16 us either way). 64^3, none
-// missing: 17 us, 26 with a CTA to copy and look through each tile; 256^3: 93
+// missing: 18 us, 26 with a CTA to copy and look through each tile; 256^3: 94
 // and 1,310.
 constexpr int kListTiles = 4;
 constexpr int kTileN = kTileX * kTileY * kTileZ;
 
-// How the solver's tiles are listed: groups of w tiles along x by v along z,
-// group (bx / w, by, bz / v) number bx / w + gx (by + ty (bz / v)). w == 0: no
-// list. The lists stand in the out entries of the plane z = 0, which are
-// written last (by the boundary kernel): words 0 to 2 are the groups with
-// missing interior entries, those with kDense or more, and the tiles the
-// solver has taken; then the groups' counts of missing interior entries, two
-// to a word, and the two lists, n words each.
+// How the solver's tiles are listed: groups of w tiles along x by v along z
+// (one tile where the list has the room), group (bx / w, by, bz / v) number
+// bx / w + gx (by + ty (bz / v)). w == 0: no list. Counts and list stand in the
+// out entries of the plane z = 0, which are written last (by the boundary
+// kernel): words 0 to 2 are the dense groups, the others with missing interior
+// entries, and the tiles the solver has taken; then the groups' counts of
+// missing interior entries, 32 >> shift bits each, and the list, n words: the
+// dense groups from its front, the others from its back.
 struct Groups {
     int tx, ty, tz;   // tiles per axis
     int w, v;
     int gx;           // groups along x
     int n;            // groups
+    int shift;        // log2 of the counts in a word
 };
-// Missing entries from which on a group counts as dense, of 128 and more: over
-// 24 lattices of 24 to 112 points an axis with losses at block faces, each with
-// two inputs, the fill takes 0.963 of the time with a CTA to each tile in
-// lattice order (0.985 at 3, 0.970 at 5, 0.972 at 12, 0.997 at 24, 1.017
-// without the order); 128^3 4.86 ms against 5.12.
+constexpr int kHead = 3;
+__host__ __device__ __forceinline__ int count_words(const Groups &G) { return ((G.n - 1) >> G.shift) + 1; }
+__device__ __forceinline__ int count_at(const Groups &G, unsigned g) {   // bit of g's count in its word
+    return (int)(g & ((1u << G.shift) - 1u)) << (5 - G.shift);
+}
+// Missing entries from which on a group is dense, for each of its tiles (of 32
+// entries). Over 24 lattices of 24 to 112 points an axis with losses at block
+// faces, two inputs each, the fill takes 0.964 of the time with a CTA to each
+// tile in lattice order (0.957 at 4, 0.963 at 12, 0.989 at 20, 1.017 without the
+// order; 128^3 4.85 ms against 5.11), over 36 lattices with random and solid
+// losses of 10% to all 1.004 (1.012, 1.010, 1.019).
 constexpr int kDense = 8;
-__host__ __device__ inline int64_t list_words(int64_t n) { return 3 + (n + 1) / 2 + 2 * n; }
 
-// Copies the valid entries (status 1), counts the groups' missing interior
-// entries and lists the groups by their first and their kDense-th. On a
-// lattice one point thick, which has no tetrahedra, the missing entries are
-// finished here. Bound by HBM: 16-byte accesses where the pointers allow it.
+// Copies the valid entries (status 1) and counts the groups' missing interior
+// entries. On a lattice one point thick, which has no tetrahedra, the missing
+// entries are finished here. Bound by HBM: 16-byte accesses where the pointers
+// allow it.
 template <bool VEC>
 __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const Groups G, bool flat,
                                                                  const float *__restrict__ ends,
@@ -1302,12 +1309,27 @@ __global__ void __launch_bounds__(kFillThreads) fill_copy_kernel(int3 S, const G
         const int x = (int)(p32 - r * (unsigned)S.x), y = (int)(r % (unsigned)S.y), z = (int)(r / (unsigned)S.y);
         if (x < 1 || x >= S.x - 1 || y < 1 || y >= S.y - 1 || z < 1 || z >= S.z - 1) continue;
         const unsigned g = (unsigned)(x / (kTileX * G.w) + G.gx * (y / kTileY + G.ty * (z / (kTileZ * G.v))));
-        unsigned *head = reinterpret_cast<unsigned *>(out), *counts = head + 3, *list = counts + (G.n + 1) / 2;
-        const int sh = (g & 1) * 16;
-        const unsigned before = atomicAdd(counts + g / 2, 1u << sh) >> sh & 0xffffu;
-        if (before == 0) list[atomicAdd(head, 1u)] = g;
-        if (before == kDense - 1) list[G.n + atomicAdd(head + 1, 1u)] = g;
+        atomicAdd(reinterpret_cast<unsigned *>(out) + kHead + (g >> G.shift), 1u << count_at(G, g));
     }
+}
+
+// Lists the groups with missing entries, a group to a thread.
+__global__ void __launch_bounds__(kFillThreads) fill_list_kernel(const Groups G, float *__restrict__ out) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the solver waits for this grid
+    unsigned *head = reinterpret_cast<unsigned *>(out), *counts = head + kHead, *list = counts + count_words(G);
+    const unsigned g = blockIdx.x * kFillThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31, bits = 32 >> G.shift;
+    const unsigned c = g < (unsigned)G.n ? __ldcg(counts + (g >> G.shift)) >> count_at(G, g) & ((1u << bits) - 1u) : 0u;
+    const unsigned some = __ballot_sync(kAll, c != 0);
+    if (!some) return;
+    const bool dense = c >= (unsigned)(kDense * G.w * G.v);
+    const unsigned front = __ballot_sync(kAll, dense), back = some & ~front;
+    unsigned at = 0;
+    if (lane < 2 && (lane ? back : front)) at = atomicAdd(head + lane, (unsigned)__popc(lane ? back : front));
+    const unsigned below = (1u << lane) - 1u, f0 = __shfl_sync(kAll, at, 0), b0 = __shfl_sync(kAll, at, 1);
+    if (dense) list[f0 + __popc(front & below)] = g;
+    else if (c) list[G.n - 1 - (b0 + __popc(back & below))] = g;
 }
 
 // Solves the missing interior entries. A CTA takes a tile: it collects the
@@ -1344,9 +1366,9 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     unsigned *head = reinterpret_cast<unsigned *>(out);
-    const unsigned *counts = head + 3, *list_of = counts + (G.n + 1) / 2;
-    const unsigned sub = (unsigned)(G.w * G.v), dense = LISTED ? __ldcg(head + 1) * sub : 0u,
-                   total = LISTED ? dense + __ldcg(head) * sub : 0u;
+    const unsigned *listed = head + kHead + count_words(G);
+    const unsigned sub = (unsigned)(G.w * G.v), front = LISTED ? __ldcg(head) : 0u,
+                   total = LISTED ? (front + __ldcg(head + 1)) * sub : 0u;
 #pragma unroll 1
     for (;;) {
         if (warp == 0) {
@@ -1355,17 +1377,16 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_interior_kernel(int3 S, 
                 unsigned job = 0, g = 0;
                 if (lane == 0) {
                     job = atomicAdd(head + 2, 1u);
-                    if (job < dense) g = __ldcg(list_of + G.n + job / sub);
-                    else if (job < total) g = __ldcg(list_of + (job - dense) / sub);
+                    const unsigned k = job / sub;
+                    if (job < total) g = __ldcg(listed + (k < front ? k : G.n - 1 - (k - front)));
                 }
                 job = __shfl_sync(kAll, job, 0);
                 g = __shfl_sync(kAll, g, 0);
-                const int in = (int)((job < dense ? job : job - dense) % sub);
+                const int in = (int)(job % sub);
                 bx = (int)(g % (unsigned)G.gx) * G.w + in % G.w;
                 by = (int)(g / (unsigned)G.gx % (unsigned)G.ty);
                 bz = (int)(g / (unsigned)G.gx / (unsigned)G.ty) * G.v + in / G.w;
                 if (job >= total) bx = -1;   // none left
-                else if (job >= dense && (__ldcg(counts + g / 2) >> (g & 1) * 16 & 0xffffu) >= kDense) bx = G.tx;   // taken
             } else {
                 bx = (int)(blockIdx.x % G.tx);
                 by = (int)(blockIdx.x / G.tx % G.ty);
@@ -1531,21 +1552,29 @@ __global__ void __launch_bounds__(kFillThreads) fill_boundary_kernel(int3 S, int
 
 BTO_BOUNDS_ACCESSOR(bounds_failures_delaunay)
 
-// The solver's groups: as few tiles along z to a group as let the lists fit
-// the plane z = 0 of out.
+// The solver's groups: as few tiles to a group as let counts and list fit the
+// plane z = 0 of out; w == 0 when none does.
 static Groups groups_of(const int32_t S[3]) {
     Groups G{};
     G.tx = (S[0] + kTileX - 1) / kTileX;
     G.ty = (S[1] + kTileY - 1) / kTileY;
     G.tz = (S[2] + kTileZ - 1) / kTileZ;
-    G.w = G.tx < 4 ? G.tx : 4;
-    G.gx = (G.tx + G.w - 1) / G.w;
-    const int64_t per = (int64_t)G.gx * G.ty, words = 3 * (int64_t)S[0] * S[1];
-    int64_t gz = (words - 4) * 2 / 5 / per;
-    if (gz > G.tz) gz = G.tz;
-    if (gz < 1) gz = 1;
-    G.v = (int)((G.tz + gz - 1) / gz);
-    G.n = (int)(per * ((G.tz + G.v - 1) / G.v));
+    const int64_t words = 3 * (int64_t)S[0] * S[1];
+    for (int size = 1; size <= 65536 / kTileN; size *= 2) {
+        G.w = size < 4 ? size : 4;
+        if (G.w > G.tx) G.w = G.tx;
+        G.v = size / G.w;
+        if (G.v > G.tz) G.v = G.tz;
+        G.gx = (G.tx + G.w - 1) / G.w;
+        const int64_t n = (int64_t)G.gx * G.ty * ((G.tz + G.v - 1) / G.v);
+        G.shift = kTileN * G.w * G.v < 256 ? 2 : 1;
+        if (kTileN * G.w * G.v >= 65536) break;
+        if (kHead + ((n - 1) >> G.shift) + 1 + n <= words) {
+            G.n = (int)n;
+            return G;
+        }
+    }
+    G.w = 0;
     return G;
 }
 
@@ -1574,11 +1603,9 @@ cudaError_t launch_fill_delaunay(const int32_t S[3], const float *ends, const ui
     const int64_t resident = 4ll * sm_count;
     const bool apart = out + 3 * P <= ends || ends + 3 * P <= out;   // the list would spoil ends
     Groups G = groups_of(S);
-    // a group's count has 16 bits
-    const bool listed = inner && apart && tiles > kListTiles * resident && list_words(G.n) <= 3 * (int64_t)S[0] * S[1] &&
-                        (int64_t)kTileN * G.w * G.v < 65536;
+    const bool listed = inner && apart && tiles > kListTiles * resident && G.w > 0;
     if (listed) {
-        const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(uint32_t) * (3 + (G.n + 1) / 2), s);
+        const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(uint32_t) * (kHead + count_words(G)), s);
         if (e != cudaSuccess) return e;
     } else {
         G.w = 0;
@@ -1592,6 +1619,8 @@ cudaError_t launch_fill_delaunay(const int32_t S[3], const float *ends, const ui
         fill_copy_kernel<false><<<copies, kFillThreads, 0, s>>>(S3, G, flat, ends, valid, out, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || flat) return e;
+    if (listed) e = launch_after(fill_list_kernel, (G.n + kFillThreads - 1) / kFillThreads, s, G, out);
+    if (e != cudaSuccess) return e;
     if (listed)
         e = launch_after(fill_interior_kernel<true>, resident, s, S3, G, ends, valid, out, status);
     else if (inner)

@@ -23,7 +23,7 @@ def test_only_the_cycle_kernels_launch_dependents_early():
     for src in glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")):
         text = re.sub(r"//[^\n]*", "", open(src).read())
         early |= _kernels_with(text, "griddepcontrol.launch_dependents")
-    within_a_call = {"fill_copy_kernel", "fill_interior_kernel"}     # fill_boundary_kernel ends the call
+    within_a_call = {"fill_copy_kernel", "fill_list_kernel", "fill_interior_kernel"}     # fill_boundary_kernel ends the call
     assert early == {"advect_kernel", "advect_tiled_kernel"} | within_a_call, early
     header = open(os.path.join(ROOT, "include", "bto.h")).read()
     assert "The cycle's kernel (here and in bto_batch_advect_cycle) is launched with" in header
